@@ -321,19 +321,21 @@ double fire_time(const fire_ctx *ctx);
  *                      rows;
  *   FIRE_KERNEL_TILE   a 2-D tile of kx*sr_x by ky*sr_y nodes staged with
  *                      a 3-node halo in shared memory (any refinement);
- *   FIRE_KERNEL_WARP   each warp marches alone down a strip of kx*sr_x
- *                      columns (an even number <= 60) and ky*sr_y rows, rows
- *                      held in registers, neighbours exchanged by shuffles;
- *   FIRE_KERNEL_WARP4  (FIRE_FP32 only) the same with four columns per lane:
- *                      strips of kx*sr_x <= 120 columns, the per-row control
- *                      shared by four columns;
- *   FIRE_KERNEL_WARP_DENSE  (FIRE_FP32 only) FIRE_KERNEL_WARP's strips
- *                      with t_i read a row ahead where psi <= 0 and the two
- *                      cells of a lane in one packed fuel-fraction
- *                      evaluation: the same results bit for bit, faster
- *                      where much of the mesh burns, slower where little
- *                      does (with a per-node moisture it runs as
- *                      FIRE_KERNEL_WARP).
+ *   FIRE_KERNEL_WARP   a CTA of four warps marches down a strip of kx*sr_x
+ *                      columns (an even number <= 60) and ky*sr_y rows, each
+ *                      warp with one row of every stage at a time, neighbours
+ *                      exchanged by shuffles and through rings of rows in
+ *                      shared memory; strips of more than 16 atmospheric rows
+ *                      are cut, and fire_init's default strips run with the
+ *                      rows per CTA that suit the mesh and the device (no
+ *                      result depends on either);
+ *   FIRE_KERNEL_WARP4  (FIRE_FP32 only) each warp marches alone down a strip
+ *                      of kx*sr_x <= 120 columns, four columns per lane, rows
+ *                      held in registers;
+ *   FIRE_KERNEL_WARP_DENSE  (FIRE_FP32 only) FIRE_KERNEL_WARP under the name
+ *                      of the choice for burning states: the same kernel (it
+ *                      reads t_i ahead where psi <= 0 and evaluates the two
+ *                      cells of a lane at once), the same results bit for bit.
  * FIRE_ERR_ARG if the shape does not fit the variant or the device. */
 enum fire_kernel_variant {
     FIRE_KERNEL_TILE = 0,

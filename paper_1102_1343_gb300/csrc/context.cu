@@ -50,6 +50,7 @@ struct fire_ctx {
 
     int variant = FIRE_KERNEL_MARCH;
     int kx = 0, ky = 0;
+    int launch_ky = 0;  // rows of a CTA of the default warp strips (0: ky)
     int scheme = 0;  // fuel fraction: 0 subcell scheme, 1 exact for linear data (tiles)
     size_t smem = 0;
     size_t smem_max = 0;
@@ -64,7 +65,7 @@ struct fire_ctx {
     const void *g_u = nullptr, *g_v = nullptr;
     double g_dt = 0;
     double *g_hs = nullptr, *g_hl = nullptr;
-    int g_kx = 0, g_ky = 0, g_variant = -1;
+    int g_kx = 0, g_ky = 0, g_launch_ky = 0, g_variant = -1;
 
     // workspace of fire_adjoint (grown on demand, freed with the context)
     void *ws = nullptr;
@@ -86,6 +87,7 @@ struct fire_ctx {
     bool adaptive = false;
     bool ad_dense = false;                       // the dense variant is chosen
     int ad_kx = 0, ad_ky = 0, ad_dense_ky = 0;   // the two shapes
+    bool ad_launch = false;                      // CTAs of warp_launch_rows (fire_init's default)
     unsigned long long *ad_count_dev = nullptr;  // nodes with psi <= 0
     unsigned long long *ad_count_host = nullptr; // page-locked copy of it
     cudaEvent_t ad_ready = nullptr;              // that copy has landed
@@ -221,7 +223,7 @@ int step_kernel_args(fire_ctx *c, const void *u, const void *v, double dt, doubl
     a.srx = c->g.sr_x;
     a.sry = c->g.sr_y;
     a.kx = c->kx;
-    a.ky = c->ky;
+    a.ky = c->launch_ky ? c->launch_ky : c->ky;
     a.band = c->g.boundary_band;
     a.dx = c->dx;
     a.dy = c->dy;
@@ -238,7 +240,7 @@ cudaError_t launch_variant(const fire_ctx *c, const StepArgs &a, cudaStream_t s)
     if (c->variant == FIRE_KERNEL_WARP4)
         return c->prec == FIRE_FP32 ? launch_warp4(a, s) : cudaErrorInvalidValue;
     if (c->variant == FIRE_KERNEL_WARP_DENSE)
-        return c->prec == FIRE_FP32 ? launch_warp<float>(a, s, true) : cudaErrorInvalidValue;
+        return c->prec == FIRE_FP32 ? launch_warp<float>(a, s) : cudaErrorInvalidValue;
     return c->prec == FIRE_FP64 ? launch_step<double>(a, s) : launch_step<float>(a, s);
 }
 
@@ -325,8 +327,11 @@ int configure_kernel(fire_ctx *c, int variant, int kx, int ky) {
         if (W > kWarpMaxColumns || (W & 1) || L > kWarpMaxRows || (long long)c->n > kWarpMaxNodes)
             return FIRE_ERR_ARG;
         if (variant == FIRE_KERNEL_WARP_DENSE && c->prec != FIRE_FP32) return FIRE_ERR_ARG;
-        sm = 0;
-        e = cudaSuccess;
+        const int kr = ky < kRowMaxBands ? ky : kRowMaxBands;
+        sm = c->prec == FIRE_FP64 ? warp_smem_bytes<double>(kr, c->g.sr_y, c->ncls)
+                                  : warp_smem_bytes<float>(kr, c->g.sr_y, c->ncls);
+        if (sm > c->smem_max) return FIRE_ERR_ARG;
+        e = c->prec == FIRE_FP64 ? prepare_warp_kernel<double>(sm) : prepare_warp_kernel<float>(sm);
     } else if (variant == FIRE_KERNEL_WARP4) {
         const long long W = (long long)kx * c->g.sr_x, L = (long long)ky * c->g.sr_y;
         if (c->prec != FIRE_FP32 || W > kWarp4MaxColumns || L > kWarpMaxRows ||
@@ -346,8 +351,15 @@ int configure_kernel(fire_ctx *c, int variant, int kx, int ky) {
     c->variant = variant;
     c->kx = kx;
     c->ky = ky;
+    c->launch_ky = 0;
     c->smem = sm;
     return FIRE_OK;
+}
+
+// the rows that a CTA takes of the default warp strips
+void default_launch_rows(fire_ctx *c) {
+    if (c->variant == FIRE_KERNEL_WARP || c->variant == FIRE_KERNEL_WARP_DENSE)
+        c->launch_ky = warp_launch_rows(c->nx, c->ny, c->kx * c->g.sr_x, c->g.sr_y, c->n_sm);
 }
 
 // marching strips of up to 248 columns (an even number) x ~60 rows
@@ -362,12 +374,12 @@ int default_march(fire_ctx *c) {
     return configure_kernel(c, FIRE_KERNEL_MARCH, kx, ky);
 }
 
-// the warp strips of the large-mesh default (~60 x 160 nodes), FP32 only
-int default_warp_strips(fire_ctx *c) {
+// warp strips of ~60 columns x `rows` rows, FP32 only
+int default_warp_strips(fire_ctx *c, int rows) {
     c->adaptive = false;  // an ensemble member keeps the ensemble's form
     if (c->prec != FIRE_FP32 || c->g.sr_x > kWarpMaxColumns / 2 || (long long)c->n > kWarpMaxNodes)
         return FIRE_ERR_ARG;
-    int kx = kWarpMaxColumns / c->g.sr_x, ky = 160 / c->g.sr_y;
+    int kx = kWarpMaxColumns / c->g.sr_x, ky = rows / c->g.sr_y;
     if (kx > c->g.nx_atm) kx = c->g.nx_atm;
     // strips of an even width; one atmospheric column at an odd refinement
     // takes a strip of two (the kernel clips a strip at the mesh edge)
@@ -380,7 +392,10 @@ int default_warp_strips(fire_ctx *c) {
 int default_kernel(fire_ctx *c) {
     const DefaultShape d = default_shape(c->prec == FIRE_FP64, c->g.nx_atm, c->g.ny_atm,
                                          c->g.sr_x, c->g.sr_y, c->n_sm);
-    if (configure_kernel(c, d.variant, d.kx, d.ky) == FIRE_OK) return FIRE_OK;
+    if (configure_kernel(c, d.variant, d.kx, d.ky) == FIRE_OK) {
+        default_launch_rows(c);
+        return FIRE_OK;
+    }
     // a strip shape whose shared memory does not fit: 2-D tiles, halved until
     // they fit
     int kx = d.variant == FIRE_KERNEL_TILE ? d.kx : (c->prec == FIRE_FP64 ? 40 : 80) / c->g.sr_x;
@@ -427,8 +442,10 @@ int adaptive_decide(fire_ctx *c, unsigned long long count) {
     if (dense == c->ad_dense) return FIRE_OK;
     const int r = configure_kernel(c, dense ? FIRE_KERNEL_WARP_DENSE : FIRE_KERNEL_WARP, c->ad_kx,
                                    dense ? c->ad_dense_ky : c->ad_ky);
-    if (r == FIRE_OK) c->ad_dense = dense;
-    return r;
+    if (r != FIRE_OK) return r;
+    c->ad_dense = dense;
+    if (c->ad_launch) default_launch_rows(c);
+    return FIRE_OK;
 }
 
 // a count and its copy to page-locked host memory, read by adaptive_update
@@ -485,6 +502,7 @@ void adaptive_setup(fire_ctx *c) {
     c->ad_dense = false;
     c->ad_kx = c->kx;
     c->ad_ky = c->ky;
+    c->ad_launch = c->launch_ky != 0;
     const int short_rows = 60 / c->g.sr_y;
     c->ad_dense_ky = c->ky < short_rows ? c->ky : (short_rows < 1 ? 1 : short_rows);
     c->ad_steps = kAdaptEvery;  // count before the first step
@@ -577,6 +595,21 @@ DefaultShape default_shape(bool fp64, int nx_atm, int ny_atm, int srx, int sry, 
     return {FIRE_KERNEL_TILE, kx, ky};
 }
 
+int warp_launch_rows(int nx, int ny, int W, int sry, int n_sm) {
+    const long strips = cdiv_l(nx, W), slots = (long)n_sm * kRowCtasPerSmF32;
+    int best = 1;
+    double least = 0;
+    for (int ky = 1; ky <= kRowMaxBands && (ky == 1 || (ky - 1) * (long)sry < ny) && (ky == 1 || ky * (long)sry <= kWarpMaxRows); ++ky) {
+        const long L = (long)ky * sry;
+        const double t = (double)(strips * cdiv_l(ny, L)) * (L + 10) / slots + 0.8 * (L + 20);
+        if (ky == 1 || t < least) {
+            least = t;
+            best = ky;
+        }
+    }
+    return best;
+}
+
 int ctx_step_args(fire_ctx *c, int parity, const void *u, const void *v, double dt, double *hs,
                   double *hl, StepArgs &a) {
     const int save = c->cur;
@@ -620,7 +653,7 @@ cudaStream_t ctx_stream(const fire_ctx *c) { return c->stream; }
 int ctx_device(const fire_ctx *c) { return c->device; }
 
 int ctx_default_march(fire_ctx *c) { return default_march(c); }
-int ctx_default_warp_strips(fire_ctx *c) { return default_warp_strips(c); }
+int ctx_default_warp_strips(fire_ctx *c, int rows) { return default_warp_strips(c, rows); }
 
 const fire_fuel_class *ctx_classes_dev(const fire_ctx *c) { return c->classes_dev; }
 const void *ctx_moisture(const fire_ctx *c) { return c->moist; }
@@ -920,7 +953,8 @@ int fire_run(fire_ctx *c, int nsteps, double dt, const void *u, const void *v, d
         if (ra) return ra;
         c->ad_steps += 2;
         if (!c->graph || c->g_u != u || c->g_v != v || c->g_dt != dt || c->g_hs != hs ||
-            c->g_hl != hl || c->g_kx != c->kx || c->g_ky != c->ky || c->g_variant != c->variant) {
+            c->g_hl != hl || c->g_kx != c->kx || c->g_ky != c->ky ||
+            c->g_launch_ky != c->launch_ky || c->g_variant != c->variant) {
             if (c->graph) {
                 WF_CHECK(cudaStreamSynchronize(c->stream));  // the old graph may be in flight
                 cudaGraphExecDestroy(c->graph);
@@ -956,6 +990,7 @@ int fire_run(fire_ctx *c, int nsteps, double dt, const void *u, const void *v, d
             c->g_hl = hl;
             c->g_kx = c->kx;
             c->g_ky = c->ky;
+            c->g_launch_ky = c->launch_ky;
             c->g_variant = c->variant;
         }
         WF_CHECK(cudaGraphLaunch(c->graph, c->stream));
@@ -1224,10 +1259,7 @@ int fire_autotune(fire_ctx *c, const void *u, const void *v, double dt, int prob
         const int heights[] = {16, 32, 64, 128, 256, 512};
         for (int W : widths) {
             if (W / srx * srx > kWarpMaxColumns || W / srx < 1) continue;
-            for (int L : heights) {
-                add(FIRE_KERNEL_WARP, W / srx, L / sry);
-                if (c->prec == FIRE_FP32) add(FIRE_KERNEL_WARP_DENSE, W / srx, L / sry);
-            }
+            for (int L : heights) add(FIRE_KERNEL_WARP, W / srx, L / sry);
         }
     }
     if (c->prec == FIRE_FP32 && srx <= kWarp4MaxColumns / 2) {

@@ -8,11 +8,9 @@
 // alone.  The launch (with the reset of the barrier word) is captured in a
 // CUDA graph and replayed while its arguments do not change.
 //
-// Two forms of the persistent kernel: FP32 ensembles run the warp-strip code
-// of k_fire_warp, one (member, strip) item per warp, each warp loading its
-// member's class table and wind-row weights into its own slice of shared
-// memory; FP64 ensembles (or refinements above 30) run the marching-strip
-// code of k_fire_march, one item per CTA.
+// Two forms of the persistent kernel, both with one (member, strip) item per
+// CTA at a time: FP32 ensembles run the strip code of k_fire_warp, FP64
+// ensembles (or refinements above 30) that of k_fire_march.
 //
 // The barrier's wait is bounded: a CTA that waits longer than the spin limit
 // sets the ensemble's TIMEOUT bit and an abort flag, and every CTA leaves the
@@ -147,29 +145,15 @@ __global__ void __launch_bounds__(kMarchThreads, MarchOccupancy<T>::blocks)
     }
 }
 
-// dynamic shared memory of the warp form: per warp a class table, the same
-// coefficients doubled for pair loads, the Hq column, heat column sums and
-// the wind-row weights of up to max_rows + 4 rows
-template <typename T>
-__host__ __device__ size_t ens_warp_slice(int max_rows) {
-    size_t b = (size_t)FIRE_MAX_CLASSES * 21 * sizeof(T) + 128 * sizeof(T);
-    b = (b + 15) & ~(size_t)15;
-    b += (size_t)(max_rows + 4) * sizeof(WRow<T>);
-    return (b + 15) & ~(size_t)15;
-}
-
+// the warp form: the CTA's warps share one item, its member's arguments in
+// shared memory
 template <typename T, bool NC>
-__global__ void __launch_bounds__(kWarpCtaThreads, WOcc<T>::blocks)
-    k_fire_ensemble_warp(const EnsembleArgs e, int max_rows) {
+__global__ void __launch_bounds__(32 * kRowWarps, (row_ctas<T, NC ? ROW_NC : ROW_MULT>()))
+    k_fire_ensemble_warp(const EnsembleArgs e) {
     extern __shared__ __align__(16) unsigned char dyn_smem[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    unsigned char *slice = dyn_smem + (size_t)warp * ens_warp_slice<T>(max_rows);
-    T *lut = reinterpret_cast<T *>(slice);
-    T *lut2 = lut + FIRE_MAX_CLASSES * 8;
-    T *lutq = lut2 + FIRE_MAX_CLASSES * 12;
-    T *hw = lutq + FIRE_MAX_CLASSES;
-    WRow<T> *rows = reinterpret_cast<WRow<T> *>(
-        slice + (((size_t)FIRE_MAX_CLASSES * 21 + 128) * sizeof(T) + 15 & ~(size_t)15));
+    __shared__ StepArgs a;
+    __shared__ int s_item;
+    RowSmem<T, kRowWarps> sm;
     const EnsRun run = *e.run;
     double t = run.t0;
     for (int s = 0; s < run.nsteps; ++s) {
@@ -178,48 +162,20 @@ __global__ void __launch_bounds__(kWarpCtaThreads, WOcc<T>::blocks)
         if (blockIdx.x == 0 && threadIdx.x == 0) e.bar->next[(s + 1) & 1] = 0;
         for (;;) {
             // items are taken dynamically, largest first (the list is sorted)
-            int i = 0;
-            if (lane == 0) i = (int)atomicAdd(&e.bar->next[s & 1], 1u);
-            i = __shfl_sync(0xffffffffu, i, 0);
+            if (threadIdx.x == 0) s_item = (int)atomicAdd(&e.bar->next[s & 1], 1u);
+            __syncthreads();
+            const int i = s_item;
             if (i >= e.n_items) break;
             const EnsItem it = e.items[i];
-            const StepArgs &a = e.margs[2 * it.member + par];
-            // the member's class table and the wind-row weights of the strip
-            for (int k = lane; k < a.ncls; k += 32) {
-                const double *co = a.coef + (size_t)k * K_N;
-                T *l = lut + k * 8;
-                l[0] = T(co[K_S0]);
-                l[1] = T(co[K_R0]);
-                l[2] = T(co[K_B]);
-                l[3] = T(co[K_C]);
-                l[4] = T(co[K_D]);
-                l[5] = T(co[K_E]);
-                l[6] = T(co[K_TF]);
-                l[7] = T(co[K_HS]);
-                lutq[k] = T(co[K_HQ]);
-                T *l2 = lut2 + k * 12;
-                for (int j = 0; j < 6; ++j) l2[2 * j] = l2[2 * j + 1] = l[j];
-            }
-            const int La = min(a.ky * a.sry, a.ny - it.y0);
-            for (int q = lane; q < La + 4; q += 32) {
-                const int r = it.y0 - 2 + q;
-                WRow<T> w;
-                w.ju0 = w.jv0 = 0;
-                w.wyu = w.wyv = T(0);
-                if (r >= 0 && r < a.ny) {
-                    int j1;
-                    const T yr = (T(r) + T(0.5)) / T(a.sry);
-                    lin_idx<T>(yr - T(0.5), a.nya, w.ju0, j1, w.wyu);
-                    lin_idx<T>(yr, a.nya + 1, w.jv0, j1, w.wyv);
-                }
-                rows[q] = w;
-            }
-            __syncwarp();
-            WarpStrip<T, NC> strip(a, lut, lut2, lutq, hw, rows);
-            strip.run(it.x0, it.y0, t);
+            const int *src = reinterpret_cast<const int *>(e.margs + 2 * it.member + par);
+            for (int q = threadIdx.x; q < (int)(sizeof(StepArgs) / sizeof(int)); q += 32 * kRowWarps)
+                reinterpret_cast<int *>(&a)[q] = src[q];
+            __syncthreads();
+            sm.carve(dyn_smem, a.ky, a.sry, a.ncls);
+            RowStrip<T, NC ? ROW_NC : ROW_MULT, kRowWarps> strip(a, sm, dyn_smem);
+            strip.run(it.x0, it.y0, t);  // ends with a barrier
             const int stw = __reduce_or_sync(0xffffffffu, strip.st);
-            if (lane == 0 && stw) atomicOr(a.status, stw);
-            __syncwarp();  // the slice is reused by the next item
+            if ((threadIdx.x & 31) == 0 && stw) atomicOr(a.status, stw);
         }
         t = t + e.dt;
         if (s + 1 < run.nsteps) {
@@ -251,7 +207,7 @@ bool ctx_ignition_active(fire_ctx *c, double t);
 cudaStream_t ctx_stream(const fire_ctx *c);
 int ctx_workspace(fire_ctx *c, size_t bytes, void **out);
 int ctx_default_march(fire_ctx *c);
-int ctx_default_warp_strips(fire_ctx *c);
+int ctx_default_warp_strips(fire_ctx *c, int rows);
 int ctx_ensure_node_coefficients(fire_ctx *c);
 bool ctx_has_node_coefficients(const fire_ctx *c);
 }  // namespace wf
@@ -278,7 +234,6 @@ struct fire_ensemble {
     bool capture_failed = false;
     int variant = FIRE_KERNEL_MARCH;  // member kernel: FIRE_KERNEL_MARCH or FIRE_KERNEL_WARP
     bool nc = false;  // members carry per-node coefficients (a per-node fuel moisture)
-    int max_rows = 0;                 // warp form: tallest strip
     int g_nsteps = -1;
     double g_dt = 0;
     int g_grid = 0;
@@ -330,12 +285,12 @@ int ens_plan(fire_ensemble *e) {
     }
     std::vector<EnsItem> items;
     size_t smem = 0;
-    int max_rows = 0;
     for (int m = 0; m < e->n; ++m) {
         int prec, variant, nx, ny, srx, sry, kx, ky, ncls, cur;
         double t;
         ctx_info(e->members[m], &prec, &variant, &nx, &ny, &srx, &sry, &kx, &ky, &ncls, &cur, &t);
         if (variant != e->variant) return FIRE_ERR_STATE;
+        if (e->variant == FIRE_KERNEL_WARP) ky = row_strip_bands(ky, sry);
         const int W = kx * srx, L = ky * sry;
         for (int y0 = 0; y0 < ny; y0 += L)
             for (int x0 = 0; x0 < nx; x0 += W) items.push_back(EnsItem{m, x0, y0});
@@ -343,12 +298,12 @@ int ens_plan(fire_ensemble *e) {
             const size_t sm = e->prec == FIRE_FP64 ? march_smem_bytes<double>(ky, sry, ncls)
                                                    : march_smem_bytes<float>(ky, sry, ncls);
             smem = std::max(smem, sm);
+        } else {
+            const size_t sm = e->prec == FIRE_FP64 ? warp_smem_bytes<double>(ky, sry, ncls)
+                                                   : warp_smem_bytes<float>(ky, sry, ncls);
+            smem = std::max(smem, sm);
         }
-        max_rows = std::max(max_rows, L);
     }
-    if (e->variant == FIRE_KERNEL_WARP)
-        smem = kWarpStrips * (e->prec == FIRE_FP64 ? ens_warp_slice<double>(max_rows)
-                                                   : ens_warp_slice<float>(max_rows));
     // largest items first (the kernel hands them out dynamically), then by
     // row and member
     std::vector<long long> cost(items.size());
@@ -357,6 +312,7 @@ int ens_plan(fire_ensemble *e) {
         double t;
         ctx_info(e->members[items[q].member], &prec, &variant, &nx, &ny, &srx, &sry, &kx, &ky,
                  &ncls, &cur, &t);
+        if (e->variant == FIRE_KERNEL_WARP) ky = row_strip_bands(ky, sry);
         cost[q] = (long long)std::min(kx * srx, nx - items[q].x0) * std::min(ky * sry, ny - items[q].y0);
     }
     std::vector<size_t> order(items.size());
@@ -385,7 +341,7 @@ int ens_plan(fire_ensemble *e) {
                           : (const void *)k_fire_ensemble_warp<float, true>)
                    : (f64 ? (const void *)k_fire_ensemble_warp<double, false>
                           : (const void *)k_fire_ensemble_warp<float, false>);
-        threads = kWarpCtaThreads;
+        threads = 32 * kRowWarps;
     } else {
         fn = e->nc ? (f64 ? (const void *)k_fire_ensemble<double, true>
                           : (const void *)k_fire_ensemble<float, true>)
@@ -411,11 +367,8 @@ int ens_plan(fire_ensemble *e) {
     ENS_CHECK(cudaGetDevice(&dev));
     ENS_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     if (per_sm < 1) return FIRE_ERR_ARG;
-    const int units = e->variant == FIRE_KERNEL_WARP ? (e->n_items + kWarpStrips - 1) / kWarpStrips
-                                                     : e->n_items;
-    e->grid = std::min(units, per_sm * sms);
+    e->grid = std::min(e->n_items, per_sm * sms);
     e->smem = smem;
-    e->max_rows = max_rows;
     return FIRE_OK;
 }
 
@@ -433,7 +386,7 @@ cudaError_t ens_launch(fire_ensemble *e, double dt, cudaStream_t s) {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof cfg);
     cfg.gridDim = dim3(e->grid);
-    cfg.blockDim = dim3(e->variant == FIRE_KERNEL_WARP ? kWarpCtaThreads : kMarchThreads);
+    cfg.blockDim = dim3(e->variant == FIRE_KERNEL_WARP ? 32 * kRowWarps : kMarchThreads);
     cfg.dynamicSmemBytes = e->smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -444,10 +397,10 @@ cudaError_t ens_launch(fire_ensemble *e, double dt, cudaStream_t s) {
     const bool f64 = e->prec == FIRE_FP64;
     if (e->variant == FIRE_KERNEL_WARP) {
         if (e->nc)
-            return f64 ? cudaLaunchKernelEx(&cfg, k_fire_ensemble_warp<double, true>, ea, e->max_rows)
-                       : cudaLaunchKernelEx(&cfg, k_fire_ensemble_warp<float, true>, ea, e->max_rows);
-        return f64 ? cudaLaunchKernelEx(&cfg, k_fire_ensemble_warp<double, false>, ea, e->max_rows)
-                   : cudaLaunchKernelEx(&cfg, k_fire_ensemble_warp<float, false>, ea, e->max_rows);
+            return f64 ? cudaLaunchKernelEx(&cfg, k_fire_ensemble_warp<double, true>, ea)
+                       : cudaLaunchKernelEx(&cfg, k_fire_ensemble_warp<float, true>, ea);
+        return f64 ? cudaLaunchKernelEx(&cfg, k_fire_ensemble_warp<double, false>, ea)
+                   : cudaLaunchKernelEx(&cfg, k_fire_ensemble_warp<float, false>, ea);
     }
     if (e->nc)
         return f64 ? cudaLaunchKernelEx(&cfg, k_fire_ensemble<double, true>, ea)
@@ -494,9 +447,10 @@ int fire_ensemble_create(fire_ensemble **out, int n_members, const fire_member_d
                 if (r == FIRE_OK) r = ctx_ensure_node_coefficients(c);
     }
     // the warp form when every member can take warp strips (FP32, refinement
-    // <= 30), else the marching form for all; members start from the
-    // large-mesh strips of that form (the persistent launch balances the
-    // items itself, whatever a member's size)
+    // <= 30), else the marching form for all; members start from marching
+    // strips of the large-mesh size, or from warp strips whose height suits
+    // the whole ensemble: the items of a step are handed out to the CTAs as
+    // warp_launch_rows' CTAs are to the SMs, so the same cost is least
     if (r == FIRE_OK) {
         bool warp = prec == FIRE_FP32;
         for (fire_ctx *c : e->members) {
@@ -506,8 +460,24 @@ int fire_ensemble_create(fire_ensemble **out, int n_members, const fire_member_d
             warp = warp && srx <= kWarpMaxColumns / 2 && (long long)nx * ny <= kWarpMaxNodes;
         }
         e->variant = warp ? FIRE_KERNEL_WARP : FIRE_KERNEL_MARCH;
+        int rows = 10, n_sm = 1;
+        double least = 0;
+        r = ens_cuda(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, e->device));
+        for (int L = 10; L <= 160; L += 10) {
+            double t = 0;
+            for (fire_ctx *c : e->members) {
+                int nx = 0, ny = 0;
+                fire_mesh_size(c, &nx, &ny);
+                t += (double)((nx + kWarpMaxColumns - 1) / kWarpMaxColumns) * ((ny + L - 1) / L);
+            }
+            t = t * (L + 10) / ((double)n_sm * kRowCtasPerSmF32) + 0.8 * (L + 20);
+            if (L == 10 || t < least) {
+                least = t;
+                rows = L;
+            }
+        }
         for (fire_ctx *c : e->members)
-            if (r == FIRE_OK && (warp ? ctx_default_warp_strips(c) : ctx_default_march(c)) != FIRE_OK)
+            if (r == FIRE_OK && (warp ? ctx_default_warp_strips(c, rows) : ctx_default_march(c)) != FIRE_OK)
                 r = FIRE_ERR_ARG;
     }
 #define ENS_TRY(call)                 \
@@ -582,6 +552,8 @@ int fire_ensemble_step(fire_ensemble *e, int nsteps, double dt, const void *cons
                                           heat_lat_dev ? heat_lat_dev[m] : nullptr,
                                           e->margs_host[2 * m + p]);
                     if (r) return r;
+                    StepArgs &ma = e->margs_host[2 * m + p];
+                    if (e->variant == FIRE_KERNEL_WARP) ma.ky = row_strip_bands(ma.ky, ma.sry);
                 }
             }
             e->run_host->t0 = t0;

@@ -130,20 +130,31 @@ cudaError_t prepare_march_kernel(size_t smem_bytes);
 constexpr int kMarchMaxColumns = 248;  // output columns of one marching strip (even)
 
 template <typename T>
-cudaError_t launch_warp(const StepArgs &a, cudaStream_t s, bool dense = false);
+size_t warp_smem_bytes(int ky, int sry, int ncls);
+
+template <typename T>
+cudaError_t prepare_warp_kernel(size_t smem_bytes);
+
+template <typename T>
+cudaError_t launch_warp(const StepArgs &a, cudaStream_t s);
 
 // four columns per lane (FP32 only): strips of <= 120 output columns
 constexpr int kWarp4MaxColumns = 120;
 cudaError_t launch_warp4(const StepArgs &a, cudaStream_t s);
 
-constexpr int kWarpStrips = 4;       // warps (strips) per CTA of the warp kernel
+constexpr int kRowWarps = 4;         // warps of a CTA of the warp kernel, one row each at a time
+constexpr int kRowCtasPerSmF32 = 6;  // its resident CTAs per SM that the registers allow
+constexpr int kRowMaxBands = 16;     // atmospheric rows of one CTA of it at most
+constexpr int kWarpStrips = 4;       // warps (strips) per CTA of the four-column warp kernel
 constexpr int kWarpMaxColumns = 60;  // output columns of one warp strip (even)
 constexpr int kWarpMaxRows = 512;    // output rows of one warp strip
 // the warp kernel indexes the mesh with 32-bit offsets: nx * ny below 2^31
 constexpr long long kWarpMaxNodes = 2147483647LL;
 
-// resident CTAs per SM of the strip kernels (the minimum blocks of their
-// __launch_bounds__, checked where the kernels are defined)
+// resident CTAs per SM that default_shape counts on: of the warp strips (four
+// strips to a CTA; the rule's own unit, the launch takes warp_launch_rows),
+// and of the marching strips (the minimum blocks of their __launch_bounds__,
+// checked where the kernels are defined)
 constexpr int kWarpCtasPerSmF32 = 3;
 constexpr int kMarchCtasPerSmF32 = 5;
 constexpr int kMarchCtasPerSmF64 = 2;
@@ -161,6 +172,16 @@ struct DefaultShape {
     int variant, kx, ky;
 };
 DefaultShape default_shape(bool fp64, int nx_atm, int ny_atm, int srx, int sry, int n_sm);
+
+// Atmospheric rows of one CTA of the warp kernel where the caller did not set
+// them (fire_init's default and fire_step_noalloc): a CTA of L rows takes
+// about L + 10 rows' time (halo rows, tables, the run-in of its stages), and
+// the last CTAs to finish leave about 0.8 (L + 20) rows' time of an emptying
+// device.  The sum of both over kRowCtasPerSmF32 CTAs per SM is least near
+// the measured best: 2000^2 nodes 30 rows (10: 100 us, 30: 64, 60: 69, 160:
+// 100), 1000^2 20 rows (10: 32 us, 20: 27, 30: 30), 510^2 10 rows (10: 14.5,
+// 20: 20).
+int warp_launch_rows(int nx, int ny, int W, int sry, int n_sm);
 
 cudaError_t launch_coefficients(const fire_fuel_class *classes_dev, int n, double *coef_dev,
                                 cudaStream_t s);

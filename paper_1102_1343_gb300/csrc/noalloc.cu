@@ -165,7 +165,7 @@ extern "C" int fire_step_noalloc(const fire_grid_desc *grid, const fire_fuel_cla
     cudaError_t e = cudaErrorInvalidValue;
     if (d.variant == FIRE_KERNEL_WARP && (long long)d.ky * g.sr_y <= kWarpMaxRows) {
         a.kx = d.kx;
-        a.ky = d.ky;
+        a.ky = warp_launch_rows(a.nx, a.ny, d.kx * g.sr_x, g.sr_y, n_sm);
         e = launch_warp<float>(a, st);
         return e == cudaSuccess ? FIRE_OK : FIRE_ERR_CUDA;
     }

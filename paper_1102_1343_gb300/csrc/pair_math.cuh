@@ -61,15 +61,26 @@ __device__ __forceinline__ double max3_val(double a, double b, double c) { retur
 
 // unit vectors of two (cx, cy): Mth::unit on pairs
 __device__ __forceinline__ void unit2(float2 cx, float2 cy, float2 &nx, float2 &ny) {
+    // 2^63 = 1/sqrt(kNormMin): where both components vanish the vector stays
+    // zero (0 times that)
     const float2 n2 = fma2(cx, cx, mul2(cy, cy));
-    const float2 r = make_float2(rsqrt_ftz(fmaxf(n2.x, Mth<float>::kNormMin)),
-                                 rsqrt_ftz(fmaxf(n2.y, Mth<float>::kNormMin)));
+    const float2 r = make_float2(fminf(rsqrt_ftz(n2.x), 9223372036854775808.0f),
+                                 fminf(rsqrt_ftz(n2.y), 9223372036854775808.0f));
     nx = mul2(cx, r);
     ny = mul2(cy, r);
 }
 __device__ __forceinline__ void unit2(double2 cx, double2 cy, double2 &nx, double2 &ny) {
     Mth<double>::unit(cx.x, cy.x, nx.x, ny.x);
     Mth<double>::unit(cx.y, cy.y, nx.y, ny.y);
+}
+
+// x^b of two columns: Mth::pw on pairs
+__device__ __forceinline__ float2 pow_pair(float2 x, float2 b) {
+    const float2 e = mul2(b, make_float2(lg2_ftz(x.x), lg2_ftz(x.y)));
+    return make_float2(ex2_ftz(e.x), ex2_ftz(e.y));
+}
+__device__ __forceinline__ double2 pow_pair(double2 x, double2 b) {
+    return make_double2(Mth<double>::pw(x.x, b.x), Mth<double>::pw(x.y, b.y));
 }
 
 // coefficients of eq. (spread-WRF-Fire) for the two columns
@@ -88,7 +99,8 @@ struct WCoef {
 // Godunov's |D| = max(D-, -D+, 0) and the Laplacian -(D-x + (-D+x)) - (...)
 // need no negated operand, and G = S (|grad psi| - eps Lap) =
 // S (|grad psi| + eps (D-x - D+x + D-y - D+y)).
-template <typename T>
+// HASM false: every multiplier is 1 (m is not read).
+template <typename T, bool HASM = true>
 __device__ __forceinline__ typename PairT<T>::t neg_rhs2(
     typename PairT<T>::t p, typename PairT<T>::t pl, typename PairT<T>::t pr,
     typename PairT<T>::t pd, typename PairT<T>::t pu, typename PairT<T>::t idx2,
@@ -108,11 +120,13 @@ __device__ __forceinline__ typename PairT<T>::t neg_rhs2(
     const V g2 = fma2(gx, gx, mul2(gy, gy));
     // central differences, zeroed at the rounding level of their values
     V ddx = sub2(pr, pl), ddy = sub2(pu, pd);
-    const T z = Mth<T>::kGradZero;
-    ddx.x = abs_val(ddx.x) <= z * (abs_val(pr.x) + abs_val(pl.x)) ? T(0) : ddx.x;
-    ddx.y = abs_val(ddx.y) <= z * (abs_val(pr.y) + abs_val(pl.y)) ? T(0) : ddx.y;
-    ddy.x = abs_val(ddy.x) <= z * (abs_val(pu.x) + abs_val(pd.x)) ? T(0) : ddy.x;
-    ddy.y = abs_val(ddy.y) <= z * (abs_val(pu.y) + abs_val(pd.y)) ? T(0) : ddy.y;
+    const V z = splat<V>(Mth<T>::kGradZero);
+    const V zx2 = mul2(z, mk2(abs_val(pr.x) + abs_val(pl.x), abs_val(pr.y) + abs_val(pl.y)));
+    const V zy2 = mul2(z, mk2(abs_val(pu.x) + abs_val(pd.x), abs_val(pu.y) + abs_val(pd.y)));
+    ddx.x = abs_val(ddx.x) <= zx2.x ? T(0) : ddx.x;
+    ddx.y = abs_val(ddx.y) <= zx2.y ? T(0) : ddx.y;
+    ddy.x = abs_val(ddy.x) <= zy2.x ? T(0) : ddy.x;
+    ddy.y = abs_val(ddy.y) <= zy2.y ? T(0) : ddy.y;
     const V cx = mul2(ddx, i2dx2), cy = mul2(ddy, i2dy2);
     V nxv, nyv;
     unit2(cx, cy, nxv, nyv);
@@ -124,12 +138,11 @@ __device__ __forceinline__ typename PairT<T>::t neg_rhs2(
     Ue.y = min_val(max_val(U.y, T(0)), co.e.y);
     tq.x = max_val(tp.x, T(0));
     tq.y = max_val(tp.y, T(0));
-    pw.x = Mth<T>::pw(Ue.x, co.b.x);
-    pw.y = Mth<T>::pw(Ue.y, co.b.y);
+    pw = pow_pair(Ue, co.b);
     V s = fma2(mul2(co.d, tq), tq, fma2(co.c, pw, co.R0));
     s.x = max_val(s.x, co.S0.x);
     s.y = max_val(s.y, co.S0.y);
-    const V S = mul2(m, s);
+    const V S = HASM ? mul2(m, s) : s;
     const V nlap = add2(add2(dxm, ndxp), add2(dym, ndyp));  // -Lap
     V grad;
     grad.x = Mth<T>::sqr(g2.x);
