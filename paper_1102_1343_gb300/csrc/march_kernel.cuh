@@ -525,17 +525,17 @@ struct MarchStrip {
         // ---- average over the band's atmospheric cells (after its last row)
         if (band_end) {
             const int kxa = Wa / srx;
-            if (c < kxa) {
+            for (int cell = c; cell < kxa; cell += NT) {
                 const T *hb = sm.HB + bpar * 4 * NT;
                 // the cell's column sums in the path precision, one
                 // conversion to double per atmospheric cell
                 T h0 = T(0), h1 = T(0);
                 for (int e = 0; e < srx; ++e) {
-                    const int lc = kMarchHalo + c * srx + e;
+                    const int lc = kMarchHalo + cell * srx + e;
                     h0 += hb[lc];
                     h1 += hb[2 * NT + lc];
                 }
-                const size_t ga = WF_CHK((size_t)(rd / sry) * nxa + (x0 / srx + c), (long long)nxa * nya, st);
+                const size_t ga = WF_CHK((size_t)(rd / sry) * nxa + (x0 / srx + cell), (long long)nxa * nya, st);
                 if (a.heat_s) a.heat_s[ga] = (double)h0 * hscale;
                 if (a.heat_l) a.heat_l[ga] = (double)h1 * hscale;
             }

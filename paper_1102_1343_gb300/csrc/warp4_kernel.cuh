@@ -598,14 +598,14 @@ struct WarpStrip4 {
                 make_float4(acc_q[0].x, acc_q[0].y, acc_q[1].x, acc_q[1].y);
             __syncwarp();
             const int cells = Wa / srx;
-            if (lane < cells) {
+            for (int c = lane; c * srx < Wa; c += 32) {  // one lane per atmospheric cell
                 float h0 = 0.0f, h1 = 0.0f;
                 for (int e = 0; e < srx; ++e) {
-                    const int lc = 4 + lane * srx + e;
+                    const int lc = 4 + c * srx + e;
                     h0 += hw[lc];
                     h1 += hw[kWarp4Cols + lc];
                 }
-                const size_t ga = (size_t)(rD / sry) * nxa + (x0 / srx + lane);
+                const size_t ga = (size_t)(rD / sry) * nxa + (x0 / srx + c);
                 if (a.heat_s) a.heat_s[ga] = (double)h0 * hscale;
                 if (a.heat_l) a.heat_l[ga] = (double)h1 * hscale;
             }
