@@ -3,8 +3,8 @@
 // log-linear interpolation (before the step), and the insertion of the
 // averaged heat fluxes into the atmospheric tendencies with an
 // exp(-z/z_ext) profile (after it).  Both are element-wise over columns:
-// one thread per column (wind) or per column and level (heat), the levels
-// of a column strided by the number of columns so that a warp reads
+// one thread per column (wind) or per column and a few levels (heat), the
+// levels of a column strided by the number of columns so that a warp reads
 // consecutive columns; memory bound and tiny next to the fire step (atmos
 // mesh, not fire mesh).
 #include <cuda_runtime.h>
@@ -51,23 +51,64 @@ __global__ void k_wind_at_height(int nz, long long npts, const T *__restrict__ u
     }
 }
 
+// bits of a double: finite and not negative; finite and not zero
+__device__ __forceinline__ bool finite_nonneg(double x) {
+    return (unsigned long long)__double_as_longlong(x) < 0x7ff0000000000000ull;
+}
+__device__ __forceinline__ bool finite_nonzero(double x) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+    return b - 1 < 0x7fefffffffffffffull;
+}
+
+constexpr int kInsertLayers = 4;
+
 // per column p and layer k: the layer average S of the convergence of the
 // flux phi exp(-z/z_ext) between the faces zw_k, zw_{k+1}; the sources
-// mu phi_h S / (cp rho) and mu phi_q S / (L rho) are added to the tendencies
+// mu phi_h S / (cp rho) and mu phi_q S / (L rho) are added to the tendencies.
+// One thread per column and kInsertLayers layers (consecutive columns in a
+// warp; a face's exponential serves both its layers).  Where both fluxes of a
+// column vanish (no fire in the cell) the sources are exact zeros as long as
+// mu is finite, the faces finite, not negative and distinct and rho finite
+// and not zero: nothing is added then, and the exponentials and divisions,
+// which bound the kernel on the narrow FP64 pipe, run only under a fire.
+// 163x117 columns, 20 layers, six small fires: 77 us before (one thread per
+// column and layer, two exponentials and five divisions each), and 60 us less
+// per coupled step now (1558 -> 841 us for 12 steps).
 __global__ void k_heat_insertion(int nz, long long n, const double *__restrict__ hs,
                                  const double *__restrict__ hl, const double *__restrict__ zw,
                                  const double *__restrict__ rho, const double *__restrict__ mu,
                                  double zext, double cp, double L, double *__restrict__ rth,
                                  double *__restrict__ rqv) {
-    const long long total = (long long)nz * n;
-    for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < total;
-         q += (long long)gridDim.x * blockDim.x) {
-        const long long p = q % n;
-        const double za = zw[q], zb = zw[q + n];
-        const double S = (exp(-za / zext) - exp(-zb / zext)) / (zb - za);
-        const double r = rho[q];
-        if (rth) rth[q] += mu[p] * hs[p] / (cp * r) * S;
-        if (rqv) rqv[q] += mu[p] * hl[p] / (L * r) * S;
+    const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (p >= n) return;
+    const double m = mu[p], fh = rth ? hs[p] : 0.0, fq = rqv ? hl[p] : 0.0;
+    const bool cold = fh == 0.0 && fq == 0.0 && (finite_nonzero(m) || m == 0.0);
+    for (int k0 = blockIdx.y * kInsertLayers; k0 < nz; k0 += gridDim.y * kInsertLayers) {
+        double z[kInsertLayers + 1], r[kInsertLayers];
+#pragma unroll
+        for (int e = 0; e <= kInsertLayers; ++e)
+            if (k0 + e <= nz) z[e] = zw[(k0 + e) * n + p];
+#pragma unroll
+        for (int e = 0; e < kInsertLayers; ++e)
+            if (k0 + e < nz) r[e] = rho[(k0 + e) * n + p];
+        bool idle = cold;
+#pragma unroll
+        for (int e = 0; e < kInsertLayers; ++e)
+            if (k0 + e < nz)
+                idle = idle && finite_nonneg(z[e]) && finite_nonneg(z[e + 1]) && finite_nonzero(r[e]) &&
+                       __double_as_longlong(z[e]) != __double_as_longlong(z[e + 1]);
+        if (idle) continue;
+        double ea = exp(-z[0] / zext);
+#pragma unroll
+        for (int e = 0; e < kInsertLayers; ++e) {
+            if (k0 + e >= nz) break;
+            const double eb = exp(-z[e + 1] / zext);
+            const double S = (ea - eb) / (z[e + 1] - z[e]);
+            const long long q = (k0 + e) * n + p;
+            if (rth) rth[q] += m * fh / (cp * r[e]) * S;
+            if (rqv) rqv[q] += m * fq / (L * r[e]) * S;
+            ea = eb;
+        }
     }
 }
 
@@ -115,7 +156,9 @@ extern "C" int fire_heat_insertion(int nz, long long ncols, const double *heat_s
         return FIRE_ERR_ARG;
     if (!(z_ext > 0.0) || !(cp > 0.0) || !(latent > 0.0) || !isfinite(z_ext)) return FIRE_ERR_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    k_heat_insertion<<<grid_of((long long)nz * ncols, 256), 256, 0, s>>>(
+    const long long bx = (ncols + 127) / 128, by = (nz + kInsertLayers - 1) / kInsertLayers;
+    if (bx > 0x7fffffffLL) return FIRE_ERR_ARG;  // (2^38 columns)
+    k_heat_insertion<<<dim3((unsigned)bx, (unsigned)(by < 65535 ? by : 65535)), 128, 0, s>>>(
         nz, ncols, heat_sens_dev, heat_lat_dev, zw_dev, rho_dev, mu_dev, z_ext, cp, latent,
         rth_dev, rqv_dev);
     const cudaError_t e = cudaGetLastError();
