@@ -102,9 +102,10 @@ struct AdjArgs {
     const T *zx, *zy, *mult;  // mult nullable (1)
     const T *u, *v;
     const T *unv;  // [n][2] node wind of the run (interpolated once), or null
-    const double *coef, *dcoef;  // [ncls][K_N], or [n][K_N] per node when nodeco
+    const double *coef, *dcoef;  // [ncls][K_N]
     int ncls;
-    int nodeco;  // coefficients per node (a per-node fuel moisture)
+    // R0, c, d and d/dM_f of them per node (a per-node fuel moisture), or null
+    const T *nco[3], *dnco[3];
     const double *tign0, *tign, *tobs;
     const double *dJdt;  // dJ/dt_i per node instead of t_i - t_obs (heat misfit), or null
     const double *tsp;  // [2] start and end time of the step (device)
@@ -148,40 +149,36 @@ struct NodeEnv {
     T m, un, vn, zx, zy;
 };
 
-// the coefficients of node k (from the class table lut, [ncls][10] in T:
-// the six coefficients, then d/dM_f of S0, R0, c, d; from the double tables
-// when lut is null or the coefficients are per node), its multiplier, slope
-// and node wind
+// the per-node coefficients of node k, where there are any, in place of its
+// class's
 template <typename T>
-__device__ __forceinline__ void node_env(const AdjArgs<T> &a, const T *lut, size_t k, bool want_d,
-                                         NodeEnv<T> &e) {
-    if (a.nodeco || !lut) {
-        size_t row = k;
-        if (!a.nodeco) {
-            const int cls = a.fuel[k];
-            row = (size_t)(cls > a.ncls - 1 ? a.ncls - 1 : cls);
-        }
-        const double *co = a.coef + row * K_N;
+__device__ __forceinline__ void node_coefs(const AdjArgs<T> &a, size_t k, bool want_d, NodeEnv<T> &e) {
+    if (!a.nco[0]) return;
+    e.co[K_R0] = a.nco[0][k];
+    e.co[K_C] = a.nco[1][k];
+    e.co[K_D] = a.nco[2][k];
+    if (want_d) {
 #pragma unroll
-        for (int q = 0; q < 6; ++q) e.co[q] = T(co[q]);
-        if (want_d) {
-            const double *dc = a.dcoef + row * K_N;
-            e.dco[0] = T(dc[K_S0]);
-            e.dco[1] = T(dc[K_R0]);
-            e.dco[2] = T(dc[K_C]);
-            e.dco[3] = T(dc[K_D]);
-        }
-    } else {
-        int cls = a.fuel[k];
-        cls = cls > a.ncls - 1 ? a.ncls - 1 : cls;
-        const T *l = lut + cls * 10;
-#pragma unroll
-        for (int q = 0; q < 6; ++q) e.co[q] = l[q];
-        if (want_d) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) e.dco[q] = l[6 + q];
-        }
+        for (int q = 0; q < 3; ++q) e.dco[1 + q] = a.dnco[q][k];
     }
+}
+
+// the coefficients of node k, its multiplier, slope and node wind
+template <typename T>
+__device__ __forceinline__ void node_env(const AdjArgs<T> &a, size_t k, bool want_d, NodeEnv<T> &e) {
+    const int cls = a.fuel[k];
+    const size_t row = (size_t)(cls > a.ncls - 1 ? a.ncls - 1 : cls);
+    const double *co = a.coef + row * K_N;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) e.co[q] = T(co[q]);
+    if (want_d) {
+        const double *dc = a.dcoef + row * K_N;
+        e.dco[0] = T(dc[K_S0]);
+        e.dco[1] = T(dc[K_R0]);
+        e.dco[2] = T(dc[K_C]);
+        e.dco[3] = T(dc[K_D]);
+    }
+    node_coefs(a, k, want_d, e);
     e.m = a.mult ? a.mult[k] : T(1);
     e.zx = a.zx[k];
     e.zy = a.zy[k];
@@ -355,7 +352,7 @@ __global__ void k_adj_stage1(const AdjArgs<T> a) {
         }
         a.mu[k] = mu;
         NodeEnv<T> e;
-        node_env<T>(a, nullptr, k, false, e);
+        node_env<T>(a, k, false, e);
         T p, pl, pr, pd, pu;
         stencil(a.pa, a.nx, a.ny, i, j, p, pl, pr, pd, pu);
         const T F = rhs_vals<T>(p, pl, pr, pd, pu, a.idx, a.idy, a.i2dx, a.i2dy, a.eps, e.co,
@@ -369,7 +366,7 @@ __global__ void k_adj_stage1(const AdjArgs<T> a) {
 template <typename T>
 __device__ __forceinline__ void vjp_node(const AdjArgs<T> &a, size_t k, int i, int j, T v) {
     NodeEnv<T> e;
-    node_env<T>(a, nullptr, k, true, e);
+    node_env<T>(a, k, true, e);
     T p, pl, pr, pd, pu;
     stencil(a.X, a.nx, a.ny, i, j, p, pl, pr, pd, pu);
     Partials<T> o;
@@ -554,26 +551,14 @@ struct RevSm {
 template <typename T>
 __device__ __forceinline__ void rev_env(const AdjArgs<T> &a, const RevSm<T> &sm, int l3, size_t k,
                                         bool want_d, NodeEnv<T> &e) {
-    if (a.nodeco) {
-        const double *co = a.coef + k * K_N;
+    const T *c = sm.lut + sm.cls[l3] * 10;
 #pragma unroll
-        for (int q = 0; q < 6; ++q) e.co[q] = T(co[q]);
-        if (want_d) {
-            const double *dc = a.dcoef + k * K_N;
-            e.dco[0] = T(dc[K_S0]);
-            e.dco[1] = T(dc[K_R0]);
-            e.dco[2] = T(dc[K_C]);
-            e.dco[3] = T(dc[K_D]);
-        }
-    } else {
-        const T *c = sm.lut + sm.cls[l3] * 10;
+    for (int q = 0; q < 6; ++q) e.co[q] = c[q];
+    if (want_d) {
 #pragma unroll
-        for (int q = 0; q < 6; ++q) e.co[q] = c[q];
-        if (want_d) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) e.dco[q] = c[6 + q];
-        }
+        for (int q = 0; q < 4; ++q) e.dco[q] = c[6 + q];
     }
+    node_coefs(a, k, want_d, e);
     e.m = sm.m[l3];
     e.zx = sm.zx[l3];
     e.zy = sm.zy[l3];
@@ -583,19 +568,21 @@ __device__ __forceinline__ void rev_env(const AdjArgs<T> &a, const RevSm<T> &sm,
 
 // the product v J_F^T at node (x, y) against X (its stencil at lx, row
 // width Wx): the five stencil contributions into the radius-2 slots at l2
-// and its parameter terms (multiplier, moisture, node wind) into g[4]
+// and, for a node of the tile (own), its parameter terms (multiplier,
+// moisture, node wind) into g[4]
 template <typename T>
 __device__ __forceinline__ void rev_vjp(const AdjArgs<T> &a, const RevSm<T> &sm, const T *X,
                                         int lx, int Wx, int l3, int l2, int x, int y, size_t k,
-                                        T v, T g[4]) {
+                                        T v, bool own, T g[4]) {
     NodeEnv<T> e;
-    rev_env(a, sm, l3, k, true, e);
+    rev_env(a, sm, l3, k, own, e);
     T p, pl, pr, pd, pu;
     rev_stencil(X, lx, Wx, x, y, a.nx, a.ny, p, pl, pr, pd, pu);
     Partials<T> o;
     node_partials<T>(p, pl, pr, pd, pu, a.idx, a.idy, a.i2dx, a.i2dy, a.eps, e, o);
 #pragma unroll
     for (int q = 0; q < 5; ++q) sm.C[q * rev_rsize(2) + l2] = v * o.dpsi[q];
+    if (!own) return;
     g[0] = v * o.dm;
     g[1] = v * (o.dS0 * e.dco[0] + o.dR0 * e.dco[1] + o.dc * e.dco[2] + o.dd * e.dco[3]);
     g[2] = v * o.dun;
@@ -643,12 +630,10 @@ __global__ void __launch_bounds__(kRevThreads) k_adj_step(const AdjArgs<T> a) {
     };
     // ---- every read from global memory (each loop loads into registers
     // first and stores to shared memory after)
-    if (!a.nodeco) {
-        for (int q = tid; q < a.ncls * 10; q += kRevThreads) {
-            const int c = q / 10, m = q % 10;
-            const int src = m < 6 ? m : (m == 6 ? K_S0 : m == 7 ? K_R0 : m == 8 ? K_C : K_D);
-            sm.lut[q] = T((m < 6 ? a.coef : a.dcoef)[(size_t)c * K_N + src]);
-        }
+    for (int q = tid; q < a.ncls * 10; q += kRevThreads) {
+        const int c = q / 10, m = q % 10;
+        const int src = m < 6 ? m : (m == 6 ? K_S0 : m == 7 ? K_R0 : m == 8 ? K_C : K_D);
+        sm.lut[q] = T((m < 6 ? a.coef : a.dcoef)[(size_t)c * K_N + src]);
     }
     {
         constexpr int I4 = rev_iters(4);
@@ -796,9 +781,10 @@ __global__ void __launch_bounds__(kRevThreads) k_adj_step(const AdjArgs<T> a) {
         if (!region(2, e, x, y)) continue;
         const int l3 = at(3, x, y), l2 = at(2, x, y);
         T g[4];
-        rev_vjp(a, sm, sm.ps, l3, W3, l3, l2, x, y, (size_t)y * nx + x, a.hdtT * sm.mu[l2], g);
         const int ox = x - x0, oy = y - y0;
-        if (ox >= 0 && ox < kRevTX && oy >= 0 && oy < kRevTY) {
+        const bool own = ox >= 0 && ox < kRevTX && oy >= 0 && oy < kRevTY;
+        rev_vjp(a, sm, sm.ps, l3, W3, l3, l2, x, y, (size_t)y * nx + x, a.hdtT * sm.mu[l2], own, g);
+        if (own) {
             const int o = oy * kRevTX + ox;
 #pragma unroll
             for (int q = 0; q < 4; ++q) sm.G[q * kRevO + o] = g[q];
@@ -821,10 +807,11 @@ __global__ void __launch_bounds__(kRevThreads) k_adj_step(const AdjArgs<T> a) {
         const size_t k = (size_t)y * nx + x;
         const int l2 = at(2, x, y);
         T g[4];
-        rev_vjp(a, sm, sm.pa, at(4, x, y), W4, at(3, x, y), l2, x, y, k,
-                a.hdtT * sm.mu[l2] + a.dtT * sm.ls[at(1, x, y)], g);
         const int ox = x - x0, oy = y - y0;
-        if (ox >= 0 && ox < kRevTX && oy >= 0 && oy < kRevTY) {
+        const bool own = ox >= 0 && ox < kRevTX && oy >= 0 && oy < kRevTY;
+        rev_vjp(a, sm, sm.pa, at(4, x, y), W4, at(3, x, y), l2, x, y, k,
+                a.hdtT * sm.mu[l2] + a.dtT * sm.ls[at(1, x, y)], own, g);
+        if (own) {
             const int o = oy * kRevTX + ox;
             const int nq = a.wind_grads ? 4 : 2;
             typename GAcc<T>::t acc[4];
@@ -937,8 +924,9 @@ struct HeatArgs {
     const T *psi, *F0, *F1;  // psi and F at the end, F at the start of the run
     const double *tign;      // t_i at the end
     const uint8_t *fuel;
-    const double *coef, *dcoef;  // [ncls][K_N], or [n][K_N] per node when nodeco
-    int nodeco;
+    const double *coef, *dcoef;  // [ncls][K_N]
+    const fire_fuel_class *classes;
+    const T *moist;  // per-node fuel moisture, or null
     int ncls, nx, ny, nxa, nya, srx, sry;
     double t1;               // model time at the end
     const double *qobs;      // [nya][nxa], NaN where unobserved
@@ -946,6 +934,19 @@ struct HeatArgs {
     double *gF, *gM;         // [n]: dJ/dF_end, moisture gradient (direct term)
     double *lamd, *dJdt;     // [n]: dJ/dpsi_end, dJ/dt_i
 };
+
+// H_s of node k, and its derivative with respect to the node's moisture
+template <typename T>
+__device__ __forceinline__ double heat_factor(const HeatArgs<T> &h, size_t k, double *d) {
+    const size_t c = (size_t)min((int)h.fuel[k], h.ncls - 1);
+    if (!h.moist) {
+        if (d) *d = h.dcoef[c * K_N + K_HS];
+        return h.coef[c * K_N + K_HS];
+    }
+    const double a = h.classes[c].fgi * h.classes[c].cmbcnst, b = 1.0 + (double)h.moist[k];
+    if (d) *d = -a / (b * b);
+    return a / b;
+}
 
 // Q and the residual per atmospheric cell (the fire cells summed row by row)
 template <typename T>
@@ -957,8 +958,7 @@ __global__ void k_heat_residual(const HeatArgs<T> h) {
         for (int j = ja * h.sry; j < (ja + 1) * h.sry; ++j)
             for (int i = ia * h.srx; i < (ia + 1) * h.srx; ++i) {
                 const size_t k = (size_t)j * h.nx + i;
-                const size_t c = h.nodeco ? k : (size_t)min((int)h.fuel[k], h.ncls - 1);
-                q += ((double)h.F0[k] - (double)h.F1[k]) * h.coef[c * K_N + K_HS];
+                q += ((double)h.F0[k] - (double)h.F1[k]) * heat_factor(h, k, nullptr);
             }
         q /= (double)(h.srx * h.sry);
         h.Q[I] = q;
@@ -976,9 +976,9 @@ __global__ void k_heat_seed(const HeatArgs<T> h) {
          k += (size_t)gridDim.x * blockDim.x) {
         const int i = (int)(k % h.nx), j = (int)(k / h.nx);
         const double r = h.res[(j / h.sry) * h.nxa + i / h.srx];
-        const size_t c = h.nodeco ? k : (size_t)min((int)h.fuel[k], h.ncls - 1);
-        h.gF[k] = -r * h.coef[c * K_N + K_HS] / r2;
-        h.gM[k] = r * ((double)h.F0[k] - (double)h.F1[k]) * h.dcoef[c * K_N + K_HS] / r2;
+        double dHs;
+        h.gF[k] = -r * heat_factor(h, k, &dHs) / r2;
+        h.gM[k] = r * ((double)h.F0[k] - (double)h.F1[k]) * dHs / r2;
     }
 }
 
@@ -1087,7 +1087,7 @@ __device__ bool heat_cell(const HeatArgs<T> &h, int i, int j, double *dw, double
             w[3 * b + a] = p;
             th[3 * b + a] = (p >= 0.0 || !((double)h.psi[kc] < 0.0)) ? h.t1 : h.tign[kc];
         }
-    const size_t c = h.nodeco ? k : (size_t)min((int)h.fuel[k], h.ncls - 1);
+    const size_t c = (size_t)min((int)h.fuel[k], h.ncls - 1);
     quad_partials(w, th, h.t1, h.coef[c * K_N + K_TF], dw, dth);
     for (int q = 0; q < 9; ++q) {
         dw[q] *= g;
@@ -1316,10 +1316,11 @@ int run_adjoint(fire_ctx *c, int nsteps, double dt, const void *u, const void *v
     const size_t o_tseg = take((K + 2) * sizeof(double));
     const size_t o_small = take(16 + kMisfitBlocks * sizeof(double) + 16);
     const size_t na = (size_t)c_nxa(c) * c_nya(c);
-    // per-node coefficients of a per-node fuel moisture ([n][K_N] doubles)
+    // a per-node fuel moisture: its coefficients are the context's planes, the
+    // derivatives of R0, c, d three planes here
     const void *moist = ctx_moisture(c);
     const bool nodeco = moist != nullptr;
-    const size_t o_nco = take(nodeco ? n * K_N * sizeof(double) : 0);
+    const size_t o_nco = take(nodeco ? 3 * n * E : 0);
     const size_t o_F0 = take(qobs ? n * E : 0);                   // F at the start (heat)
     const size_t o_Qr = take(qobs ? 2 * na * sizeof(double) : 0);  // Q, residual (heat)
     const size_t o_lam = take(2 * n * E);  // lambda^{s+1}, lambda^s
@@ -1330,7 +1331,7 @@ int run_adjoint(fire_ctx *c, int nsteps, double dt, const void *u, const void *v
     const size_t o_g = take(4 * n * sizeof(double));
     const size_t o_unv = take(2 * n * E);
     const size_t nu = (size_t)c_nya(c) * (c_nxa(c) + 1), nv = (size_t)(c_nya(c) + 1) * c_nxa(c);
-    const size_t o_dco = take(sizeof(double) * K_N * (nodeco ? n : (size_t)ncls));
+    const size_t o_dco = take(sizeof(double) * K_N * (size_t)ncls);
     const size_t o_wind = take(sizeof(double) * (nu + nv));
     const size_t o_hs = take(qobs ? 3 * n * sizeof(double) : 0);  // dJ/dF, dJ/dpsi, dJ/dt_i
     void *wsv = nullptr;
@@ -1392,15 +1393,6 @@ int run_adjoint(fire_ctx *c, int nsteps, double dt, const void *u, const void *v
     StepArgs sa;
     ctx_step_args(c, cur, u, v, dt, nullptr, nullptr, sa);
     ADJ_CHECK(cudaMemcpyAsync(tign0, sa.tign, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
-    // the coefficients the adjoint kernels read: per class, or per node
-    const double *coef_rows = sa.coef;
-    if (nodeco) {
-        double *aos = reinterpret_cast<double *>(ws + o_nco);
-        T *none[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
-        ADJ_CHECK(launch_node_coefficients<T>(ctx_classes_dev(c), ncls, sa.fuel, moist, n, none,
-                                              aos, st));
-        coef_rows = aos;
-    }
     T *F0 = reinterpret_cast<T *>(ws + o_F0);
     if (qobs) ADJ_CHECK(cudaMemcpyAsync(F0, sa.F_in, n * E, cudaMemcpyDeviceToDevice, st));
     ADJ_CHECK(cudaMemcpyAsync(tdev, times.data(), (nsteps + 1) * sizeof(double),
@@ -1481,8 +1473,9 @@ int run_adjoint(fire_ctx *c, int nsteps, double dt, const void *u, const void *v
         h.F1 = static_cast<const T *>(fin.F_in);
         h.tign = tign_final;
         h.fuel = sa.fuel;
-        h.coef = coef_rows;
-        h.nodeco = nodeco ? 1 : 0;
+        h.coef = sa.coef;
+        h.classes = ctx_classes_dev(c);
+        h.moist = static_cast<const T *>(moist);
         h.ncls = ncls;
         h.nx = nx;
         h.ny = ny;
@@ -1519,14 +1512,15 @@ int run_adjoint(fire_ctx *c, int nsteps, double dt, const void *u, const void *v
     ADJ_CHECK(cudaMemsetAsync(gm, 0, 4 * n * sizeof(double), st));
     ADJ_CHECK(cudaMemsetAsync(Fs, 0, 2 * n * E, st));
 
-    // d(coefficients)/d(M_f) per class at the class moisture, or per node at
+    // d(coefficients)/d(M_f) per class at the class moisture, and per node at
     // the node's moisture
     double *dcoef = reinterpret_cast<double *>(ws + o_dco);
-    if (nodeco)
-        ADJ_CHECK(launch_node_coefficients_dMf<T>(ctx_classes_dev(c), ncls, sa.fuel, moist, n,
-                                                  dcoef, st));
-    else
-        ADJ_CHECK(launch_coefficients_dMf(ctx_classes_dev(c), ncls, dcoef, st));
+    ADJ_CHECK(launch_coefficients_dMf(ctx_classes_dev(c), ncls, dcoef, st));
+    T *dnco[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
+    if (nodeco) {
+        for (int q = 0; q < 3; ++q) dnco[q] = reinterpret_cast<T *>(ws + o_nco) + (size_t)q * n;
+        ADJ_CHECK(launch_node_coefficients<T>(ctx_classes_dev(c), ncls, sa.fuel, moist, n, dnco, true, st));
+    }
 
     AdjArgs<T> a;
     memset(&a, 0, sizeof a);
@@ -1536,9 +1530,12 @@ int run_adjoint(fire_ctx *c, int nsteps, double dt, const void *u, const void *v
     a.mult = static_cast<const T *>(sa.mult);
     a.u = static_cast<const T *>(u);
     a.v = static_cast<const T *>(v);
-    a.coef = coef_rows;
+    a.coef = sa.coef;
     a.dcoef = dcoef;
-    a.nodeco = nodeco ? 1 : 0;
+    for (int q = 0; q < 3; ++q) {
+        a.nco[q] = nodeco ? static_cast<const T *>(sa.nco[q]) : nullptr;
+        a.dnco[q] = dnco[q];
+    }
     a.ncls = ncls;
     a.tign0 = tign0;
     a.tign = tign_final;

@@ -170,12 +170,12 @@ int build_node_coefficients(fire_ctx *c) {
         double *pl[5];
         for (int q = 0; q < 5; ++q) pl[q] = static_cast<double *>(c->nco[q]);
         WF_CHECK(launch_node_coefficients<double>(c->classes_dev, c->ncls, c->fuel, c->moist, N,
-                                                  pl, nullptr, c->stream));
+                                                  pl, false, c->stream));
     } else {
         float *pl[5];
         for (int q = 0; q < 5; ++q) pl[q] = static_cast<float *>(c->nco[q]);
         WF_CHECK(launch_node_coefficients<float>(c->classes_dev, c->ncls, c->fuel, c->moist, N,
-                                                 pl, nullptr, c->stream));
+                                                 pl, false, c->stream));
     }
     return FIRE_OK;
 }

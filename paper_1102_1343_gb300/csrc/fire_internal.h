@@ -191,17 +191,12 @@ cudaError_t launch_coefficients_dMf(const fire_fuel_class *classes_dev, int n, d
                                     cudaStream_t s);
 
 // per-node coefficients at a per-node moisture (null: class moisture):
-// planes is a host array of 5 device pointers (R0, c, d, H_s, H_q, each [n]
-// in the path precision); aos (nullable) receives [n][K_N] doubles
+// planes is a host array of device pointers, each [n] in the path precision:
+// R0, c, d, H_s, H_q, or (deriv) d/d(M_f) of R0, c, d
 template <typename T>
 cudaError_t launch_node_coefficients(const fire_fuel_class *classes_dev, int ncls,
                                      const uint8_t *fuel, const void *moist, size_t n,
-                                     T *const *planes, double *aos, cudaStream_t s);
-// d(coefficients)/d(M_f) per node at the node's moisture: [n][K_N] doubles
-template <typename T>
-cudaError_t launch_node_coefficients_dMf(const fire_fuel_class *classes_dev, int ncls,
-                                         const uint8_t *fuel, const void *moist, size_t n,
-                                         double *daos, cudaStream_t s);
+                                     T *const *planes, bool deriv, cudaStream_t s);
 
 // a fuel class fire_init accepts: a positive weight (burn time), and for a
 // Rothermel class with fuel (Table 2) a positive surface-area-to-volume

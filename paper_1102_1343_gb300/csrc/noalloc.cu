@@ -7,7 +7,7 @@
 // allocator from their time loop (an allocation there can synchronise the
 // device or fail once the pool owns the memory).  This entry point serves
 // them: the caller passes every input and output buffer, and the few
-// intermediate values the step needs (the fuel-class table, its spread-rate
+// intermediate values the step needs (the fuel classes' spread-rate
 // coefficients, the step's start and end time and, when the caller passes
 // none, the status word) live in one file-scope __device__ array of fixed
 // size instead of a cudaMalloc'ed buffer.  It launches the same kernels as
@@ -19,9 +19,11 @@
 
 #include <mutex>
 
+#include "coeffs.cuh"
 #include "fire_internal.h"
 
 using namespace wf;
+using namespace wf::coefs;
 
 namespace {
 
@@ -29,13 +31,12 @@ constexpr int kNoAllocMaxClasses = FIRE_MAX_CLASSES;
 constexpr int kMaxDevices = 64;
 
 struct NoAllocScratch {
-    fire_fuel_class classes[kNoAllocMaxClasses];
     double coef[kNoAllocMaxClasses * K_N];
     double t[2];
     int status;
 };
 
-// The scratch of every call on a device: about 11 KB, held by each device
+// The scratch of every call on a device: about 5 KB, held by each device
 // that loads the library until the process exits.  Host code must not take
 // its address directly (that is a host-side stand-in); it asks the runtime.
 static __device__ __align__(256) unsigned char g_fire_noalloc_scratch[sizeof(NoAllocScratch)];
@@ -67,12 +68,17 @@ struct SetupArgs {
     int clear_status;
 };
 
-// copies the class table (passed by value) and the start time into the
-// scratch, and clears the scratch status word when it is the one in use
-__global__ void k_noalloc_setup(const SetupArgs p, NoAllocScratch *s) {
-    const int k = threadIdx.x;
-    if (k < p.n) s->classes[k] = p.classes[k];
-    if (k == 0) {
+// the class table (passed by value), its coefficients (eight lanes per class)
+// and the start time into the scratch, and the scratch status word cleared
+// when it is the one in use
+__global__ void __launch_bounds__(8 * kNoAllocMaxClasses) k_noalloc_setup(const SetupArgs p, NoAllocScratch *s) {
+    const int k = threadIdx.x >> 3;
+    double co[K_N];
+    class_chain<double>(p.classes, p.n, co, [](double m) { return m; });
+    if ((threadIdx.x & 7) == 0 && k < p.n) {
+        for (int q = 0; q < K_N; ++q) s->coef[k * K_N + q] = co[q];
+    }
+    if (threadIdx.x == 0) {
         s->t[0] = p.t;
         if (p.clear_status) s->status = 0;
     }
@@ -118,10 +124,8 @@ extern "C" int fire_step_noalloc(const fire_grid_desc *grid, const fire_fuel_cla
     sa.n = n_classes;
     sa.t = t;
     sa.clear_status = status_dev ? 0 : 1;
-    k_noalloc_setup<<<1, kNoAllocMaxClasses, 0, st>>>(sa, s);
+    k_noalloc_setup<<<1, (8 * n_classes + 31) / 32 * 32, 0, st>>>(sa, s);
     if (cudaGetLastError() != cudaSuccess) return FIRE_ERR_CUDA;
-    if (launch_coefficients(s->classes, n_classes, s->coef, st) != cudaSuccess)
-        return FIRE_ERR_CUDA;
 
     StepArgs a;
     memset(&a, 0, sizeof a);
