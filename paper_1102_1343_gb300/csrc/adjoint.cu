@@ -186,6 +186,19 @@ __device__ __forceinline__ void node_env(const AdjArgs<T> &a, size_t k, bool wan
     e.vn = a.unv[2 * k + 1];
 }
 
+// max{x, 0}, the smaller and the order of numbers that are not negative (FP64:
+// on the bits)
+__device__ __forceinline__ float pos_val(float x) { return x > 0.0f ? x : 0.0f; }
+__device__ __forceinline__ double pos_val(double x) { return pos64(x); }
+__device__ __forceinline__ float min_pos(float a, float b) { return a < b ? a : b; }
+__device__ __forceinline__ double min_pos(double a, double b) { return min_nn(a, b); }
+__device__ __forceinline__ bool gt_nn(float a, float b) { return a > b; }
+__device__ __forceinline__ bool gt_nn(double a, double b) {
+    return (unsigned long long)__double_as_longlong(a) > (unsigned long long)__double_as_longlong(b);
+}
+__device__ __forceinline__ bool gt0(float x) { return x > 0.0f; }
+using wf::gt0;
+
 // Partial derivatives of the right-hand side of eq. (F-disc) at one node,
 // F = -S |grad psi| + eps S Lap psi with S = m max{S0, R0 + c Ue^b + d tp^2},
 // with respect to the five stencil values and to m, S0, R0, c, d and the
@@ -203,42 +216,66 @@ __device__ __forceinline__ void node_partials(T p, T pl, T pr, T pd, T pu, T idx
                                               Partials<T> &o) {
     const T dxm = (p - pl) * idx, dxp = (pr - p) * idx;
     const T dym = (p - pd) * idy, dyp = (pu - p) * idy;
-    const T ax = dxm > T(0) ? dxm : T(0), bx = dxp < T(0) ? dxp : T(0);
-    const T ay = dym > T(0) ? dym : T(0), by = dyp < T(0) ? dyp : T(0);
-    const bool xm = ax * ax > bx * bx;  // D- taken along x (else D+)
-    const bool ym = ay * ay > by * by;
-    const T gx = xm ? ax : bx, gy = ym ? ay : by;
+    T gx, gy, cx, cy, nxv, nyv, rc = T(0);
+    bool xm, ym, kx, ky, normal;  // D- taken along x, y (else D+); differences not zeroed; a normal
+    if constexpr (sizeof(T) == 8) {
+        // the branches decided on the bits (no compare on the FP64 pipe)
+        const T ax = pos64(dxm), bx = pos64(-dxp), ay = pos64(dym), by = pos64(-dyp);
+        xm = gt_nn(ax, bx);
+        ym = gt_nn(ay, by);
+        gx = xm ? ax : -bx;
+        gy = ym ? ay : -by;
+        cx = rounding_zero64(pr - pl, pr, pl);
+        cy = rounding_zero64(pu - pd, pu, pd);
+        kx = nonzero(cx);
+        ky = nonzero(cy);
+        cx *= i2dx;
+        cy *= i2dy;
+        const T cn2 = fma(cx, cx, cy * cy);
+        normal = __double2hiint(cn2) >= 0x00200000;
+        if (normal) rc = rsqrt64(cn2);
+        nxv = cx * rc;
+        nyv = cy * rc;
+    } else {
+        const T ax = dxm > T(0) ? dxm : T(0), bx = dxp < T(0) ? dxp : T(0);
+        const T ay = dym > T(0) ? dym : T(0), by = dyp < T(0) ? dyp : T(0);
+        xm = ax * ax > bx * bx;
+        ym = ay * ay > by * by;
+        gx = xm ? ax : bx;
+        gy = ym ? ay : by;
+        // central differences, zeroed at the rounding level as in the forward
+        T ddx = pr - pl, ddy = pu - pd;
+        kx = !(abs_val(ddx) <= Mth<T>::kGradZero * (abs_val(pr) + abs_val(pl)));
+        ky = !(abs_val(ddy) <= Mth<T>::kGradZero * (abs_val(pu) + abs_val(pd)));
+        ddx = kx ? ddx : T(0);
+        ddy = ky ? ddy : T(0);
+        cx = ddx * i2dx;
+        cy = ddy * i2dy;
+        Mth<T>::unit(cx, cy, nxv, nyv);
+        const T cn2 = cx * cx + cy * cy;
+        normal = cn2 > Mth<T>::kNormMin;
+        if (normal) rc = Mth<T>::rsq(cn2);
+    }
     const T grad = Mth<T>::sqr(gx * gx + gy * gy);
-    // central differences, zeroed at the rounding level as in the forward
-    T ddx = pr - pl, ddy = pu - pd;
-    const bool kx = !(abs_val(ddx) <= Mth<T>::kGradZero * (abs_val(pr) + abs_val(pl)));
-    const bool ky = !(abs_val(ddy) <= Mth<T>::kGradZero * (abs_val(pu) + abs_val(pd)));
-    ddx = kx ? ddx : T(0);
-    ddy = ky ? ddy : T(0);
-    const T cx = ddx * i2dx, cy = ddy * i2dy;
-    T nxv, nyv;
-    Mth<T>::unit(cx, cy, nxv, nyv);
-    const T cn2 = cx * cx + cy * cy;
     const T U = e.un * nxv + e.vn * nyv;
     const T tp = e.zx * nxv + e.zy * nyv;
     // spread rate and its branches
-    const T Up = U > T(0) ? U : T(0);
-    const T Ue = Up < e.co[K_E] ? Up : e.co[K_E];
-    const T tpp = tp > T(0) ? tp : T(0);
+    const T Ue = min_pos(pos_val(U), e.co[K_E]);
+    const T tpp = pos_val(tp);
     const T pwv = Mth<T>::pw(Ue, e.co[K_B]);
     const T inner = e.co[K_R0] + e.co[K_C] * pwv + e.co[K_D] * tpp * tpp;
-    const bool active = inner > e.co[K_S0];
+    const bool active = gt_nn(inner, e.co[K_S0]);
     const T St = active ? inner : e.co[K_S0];
     const T S = e.m * St;
     const T lap = (dxp - dxm) + (dyp - dym);
     const T Fs = -grad + eps * lap;  // dF/dS
-    const T dSt_dU =
-        (active && U > T(0) && U < e.co[K_E]) ? Mth<T>::dv(e.co[K_C] * e.co[K_B] * pwv, Ue) : T(0);
-    const T dSt_dT = (active && tp > T(0)) ? T(2) * e.co[K_D] * tp : T(0);
+    const T dSt_dU = (active && gt0(U) && gt_nn(e.co[K_E], pos_val(U)))
+                         ? Mth<T>::dv(e.co[K_C] * e.co[K_B] * pwv, Ue)
+                         : T(0);
+    const T dSt_dT = (active && gt0(tp)) ? T(2) * e.co[K_D] * tp : T(0);
     // the unit normal n = c/|c|: dn/dc = (I - n n^T)/|c|
     T dS_dcx = T(0), dS_dcy = T(0);
-    if (cn2 > Mth<T>::kNormMin) {
-        const T rc = Mth<T>::rsq(cn2);
+    if (normal) {
         const T dU_dcx = (e.un - U * nxv) * rc, dU_dcy = (e.vn - U * nyv) * rc;
         const T dT_dcx = (e.zx - tp * nxv) * rc, dT_dcy = (e.zy - tp * nyv) * rc;
         dS_dcx = e.m * (dSt_dU * dU_dcx + dSt_dT * dT_dcx);
@@ -247,8 +284,8 @@ __device__ __forceinline__ void node_partials(T p, T pl, T pr, T pd, T pu, T idx
     const T dcx = kx ? i2dx : T(0), dcy = ky ? i2dy : T(0);
     // d|grad|/d(one-sided differences) through the taken branch
     T wx = T(0), wy = T(0);
-    if (grad > T(0)) {
-        const T rg = Mth<T>::dv(T(1), grad);
+    if (gt0(grad)) {
+        const T rg = Mth<T>::rcp(grad);
         wx = gx * rg;
         wy = gy * rg;
     }

@@ -9,6 +9,7 @@
 #include <stdint.h>
 
 #include "fire_internal.h"
+#include "fp64_math.cuh"
 
 namespace wf {
 
@@ -84,6 +85,7 @@ struct Mth<float> {
     static __device__ __forceinline__ float pw(float x, float b) { return ex2_ftz(b * lg2_ftz(x)); }
     static __device__ __forceinline__ float ex(float x) { return __expf(x); }
     static __device__ __forceinline__ float dv(float a, float b) { return __fdividef(a, b); }
+    static __device__ __forceinline__ float rcp(float x) { return __fdividef(1.0f, x); }
     // 1 - a/b as one fused multiply-add with the hardware reciprocal (the
     // same rounding wherever it is formed, scalar or packed; b a normal
     // float, as __fdividef wants it)
@@ -106,29 +108,28 @@ struct Mth<float> {
 template <>
 struct Mth<double> {
     static constexpr double kGradZero = 1e-9;
-    static constexpr double kNormMin = 0.0;
-    // x^b for x >= 0 and b > 0 as 2^(b log2 x): fewer FP64 instructions than
-    // pow (this part's FP64 pipe bounds the FP64 step), within a few units
-    // of 1e-16 relative for the wind speeds and exponents of the model;
-    // x^b = 0 at x = 0 (the capped wind component on the upwind side of the
-    // front) skips the call, and warps whose nodes all face away from the
-    // wind skip it entirely
-    static __device__ __forceinline__ double pw(double x, double b) {
-        return x > 0.0 ? exp2(b * log2(x)) : 0.0;
-    }
+    static constexpr double kNormMin = 4.4501477170144028e-308;  // 2^-1021: below it the normal is 0
+    // x^b for x >= 0 (0 at 0: the capped wind component on the upwind side of
+    // the front; warps whose nodes all face away from the wind skip the power)
+    static __device__ __forceinline__ double pw(double x, double b) { return wind_power64(x, b); }
     static __device__ __forceinline__ double ex(double x) { return exp(x); }
-    static __device__ __forceinline__ double dv(double a, double b) { return a / b; }
+    static __device__ __forceinline__ double rcp(double x) { return rcp64(x); }
+    // a/b for a normal b: the quotient by the reciprocal, corrected once
+    static __device__ __forceinline__ double dv(double a, double b) {
+        const double y = rcp64(b), q = a * y;
+        return fma(fma(-b, q, a), y, q);
+    }
     static __device__ __forceinline__ double one_minus_div(double a, double b) {
         return 1.0 - a / b;
     }
-    static __device__ __forceinline__ double sqr(double x) { return sqrt(x); }
-    static __device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
+    static __device__ __forceinline__ double sqr(double x) { return sqrt64(x); }
+    static __device__ __forceinline__ double rsq(double x) { return rsqrt64(x); }
     // unit vector of (cx, cy) (the reciprocal square root of the squared
     // norm, two products); zero vector when the norm vanishes
     static __device__ __forceinline__ void unit(double cx, double cy, double &nx, double &ny) {
-        const double n2 = cx * cx + cy * cy;
-        if (n2 > 0.0) {
-            const double r = rsqrt(n2);
+        const double n2 = fma(cx, cx, cy * cy);
+        if (__double2hiint(n2) >= 0x00200000) {
+            const double r = rsqrt64(n2);
             nx = cx * r;
             ny = cy * r;
         } else {
@@ -150,6 +151,19 @@ __device__ __forceinline__ bool finite_val(float x) {
 __device__ __forceinline__ bool finite_val(double x) {
     return (__double_as_longlong(x) & 0x7ff0000000000000LL) != 0x7ff0000000000000LL;
 }
+
+// a set sign among three numbers (FP64: no instruction of the narrow pipe)
+__device__ __forceinline__ bool any_sign(double a, double b, double c) {
+    return (__double2hiint(a) | __double2hiint(b) | __double2hiint(c)) < 0;
+}
+__device__ __forceinline__ bool any_sign(float a, float b, float c) {
+    return (__float_as_int(a) | __float_as_int(b) | __float_as_int(c)) < 0;
+}
+__device__ __forceinline__ bool nonzero(float x) { return x != 0.0f; }
+__device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
+// x <= 0
+__device__ __forceinline__ bool le0(float x) { return x <= 0.0f; }
+__device__ __forceinline__ bool le0(double x) { return __double_as_longlong(x) <= 0; }
 
 // extrapolated ghost value beyond the last node p0 (p1 the one before it),
 // Sect. 3.1: max{p0 + (p0 - p1), p0, p1}
@@ -282,9 +296,14 @@ template <typename T>
 __device__ __forceinline__ T cell_fraction_vals(T p00, T p01, T p02, T p10, T p11, T p12, T p20,
                                                 T p21, T p22, T d00, T d01, T d02, T d10, T d11,
                                                 T d12, T d20, T d21, T d22, T Tf) {
-    T mn = min_val(min_val(min_val(p00, p01), min_val(p02, p10)),
-                   min_val(min_val(p11, p12), min_val(min_val(p20, p21), p22)));
-    if (mn >= T(0)) return T(1);  // no vertex burning: every beta is 0 exactly
+    // no vertex burning: every beta is 0 exactly (FP64: the test on the signs)
+    if constexpr (sizeof(T) == 8) {
+        if (!any_sign(p00, p01, p02) && !any_sign(p10, p11, p12) && !any_sign(p20, p21, p22)) return T(1);
+    } else {
+        T mn = min_val(min_val(min_val(p00, p01), min_val(p02, p10)),
+                       min_val(min_val(p11, p12), min_val(min_val(p20, p21), p22)));
+        if (mn >= T(0)) return T(1);
+    }
     const T h = T(0.5), q = T(0.25);
     // edge midpoints W, E, S, N and corners SW, SE, NW, NE
     T pW = h * (p10 + p11), pE = h * (p11 + p12), pS = h * (p01 + p11), pN = h * (p11 + p21);

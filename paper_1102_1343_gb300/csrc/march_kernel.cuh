@@ -244,10 +244,17 @@ struct MarchStrip {
         const T2 ub = sm.UX[(ju1 & 3) * kMarchThreads + c];
         const T2 va = sm.VX[(w.jv0 & 3) * kMarchThreads + c];
         const T2 vb = sm.VX[(jv1 & 3) * kMarchThreads + c];
-        un.x = (T(1) - w.wyu) * ua.x + w.wyu * ub.x;
-        un.y = (T(1) - w.wyu) * ua.y + w.wyu * ub.y;
-        vn.x = (T(1) - w.wyv) * va.x + w.wyv * vb.x;
-        vn.y = (T(1) - w.wyv) * va.y + w.wyv * vb.y;
+        if constexpr (sizeof(T) == 8) {
+            un.x = fma(w.wyu, ub.x - ua.x, ua.x);
+            un.y = fma(w.wyu, ub.y - ua.y, ua.y);
+            vn.x = fma(w.wyv, vb.x - va.x, va.x);
+            vn.y = fma(w.wyv, vb.y - va.y, va.y);
+        } else {
+            un.x = (T(1) - w.wyu) * ua.x + w.wyu * ub.x;
+            un.y = (T(1) - w.wyu) * ua.y + w.wyu * ub.y;
+            vn.x = (T(1) - w.wyv) * va.x + w.wyv * vb.x;
+            vn.y = (T(1) - w.wyv) * va.y + w.wyv * vb.y;
+        }
     }
 
     // the 5-point values of both columns of the thread at row r from ring
@@ -347,7 +354,7 @@ struct MarchStrip {
                 T2 PN = fma2(ndth2, add2(f1v, F2), p0v);
                 PN.x = m_s2[0] ? PN.x : T(0);
                 PN.y = m_s2[1] ? PN.y : T(0);
-                bool need[2] = {m_s2[0] && PN.x <= T(0), m_s2[1] && PN.y <= T(0)};
+                bool need[2] = {m_s2[0] && le0(PN.x), m_s2[1] && le0(PN.y)};
                 if (own_row) {
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
@@ -411,14 +418,12 @@ struct MarchStrip {
                     p[b][3] = sm.SQ[sl[b] * NT + c + 1].x;
                 }
             }
-            T vmin[4];
-#pragma unroll
-            for (int h = 0; h < 4; ++h) vmin[h] = min_val(min_val(p[0][h], p[1][h]), p[2][h]);
-            const T mid = min_val(vmin[1], vmin[2]);
-            const T mn0 = min_val(vmin[0], mid), mn1 = min_val(mid, vmin[3]);
+            // (a set sign: psi < 0 or -0, for which the quadrature gives 1 too)
+            const bool burning = any_sign(p[0][0], p[1][0], p[2][0]) || any_sign(p[0][1], p[1][1], p[2][1]) ||
+                                 any_sign(p[0][2], p[1][2], p[2][2]) || any_sign(p[0][3], p[1][3], p[2][3]);
             const bool edge = xa <= 0 || xa + 1 >= nx - 1 || rd == 0 || rd == ny - 1;
             T Fn[2] = {T(1), T(1)};
-            if (mn0 < T(0) || mn1 < T(0) || edge) {
+            if (burning || edge) {
                 T d[3][4];
                 const int sl[3] = {s2, s3, s0};
 #pragma unroll
@@ -490,11 +495,11 @@ struct MarchStrip {
             // heat flux densities, only in warps where some fuel burned
             const T dF0 = m_out[0] ? Fcur.x - Fn[0] : T(0);
             const T dF1 = m_out[1] ? Fcur.y - Fn[1] : T(0);
-            if (__any_sync(__activemask(), dF0 != T(0) || dF1 != T(0))) {
+            if (__any_sync(__activemask(), nonzero(dF0) || nonzero(dF1))) {
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
                     const T dF = j == 0 ? dF0 : dF1;
-                    if (dF != T(0)) {
+                    if (nonzero(dF)) {
                         if constexpr (NC) {
                             acc_s[j] += dF * static_cast<const T *>(a.nco[3])[WF_CHK(g + j, (long long)nx * ny, st)];
                             acc_q[j] += dF * static_cast<const T *>(a.nco[4])[WF_CHK(g + j, (long long)nx * ny, st)];

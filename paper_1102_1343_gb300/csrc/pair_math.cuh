@@ -109,6 +109,14 @@ __device__ __forceinline__ typename PairT<T>::t neg_rhs2(
     typename PairT<T>::t un, typename PairT<T>::t vn, typename PairT<T>::t zx,
     typename PairT<T>::t zy) {
     using V = typename PairT<T>::t;
+    if constexpr (sizeof(T) == 8) {
+        V g;
+        g.x = neg_rhs64<HASM>(p.x, pl.x, pr.x, pd.x, pu.x, idx2.x, idy2.x, i2dx2.x, i2dy2.x, eps2.x, co.S0.x,
+                              co.R0.x, co.b.x, co.c.x, co.d.x, co.e.x, m.x, un.x, vn.x, zx.x, zy.x);
+        g.y = neg_rhs64<HASM>(p.y, pl.y, pr.y, pd.y, pu.y, idx2.x, idy2.x, i2dx2.x, i2dy2.x, eps2.x, co.S0.y,
+                              co.R0.y, co.b.y, co.c.y, co.d.y, co.e.y, m.y, un.y, vn.y, zx.y, zy.y);
+        return g;
+    }
     const V dxm = mul2(sub2(p, pl), idx2), ndxp = mul2(sub2(p, pr), idx2);
     const V dym = mul2(sub2(p, pd), idy2), ndyp = mul2(sub2(p, pu), idy2);
     // Godunov (eq. Godunov): |D| = max(D-, -D+, 0) per direction
