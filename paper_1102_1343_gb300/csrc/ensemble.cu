@@ -146,9 +146,11 @@ __global__ void __launch_bounds__(kMarchThreads, MarchOccupancy<T>::blocks)
 }
 
 // the warp form: the CTA's warps share one item, its member's arguments in
-// shared memory
-template <typename T, bool NC>
-__global__ void __launch_bounds__(32 * kRowWarps, (row_ctas<T, NC ? ROW_NC : ROW_MULT>()))
+// shared memory.  One CTA per SM fewer than k_fire_warp: at 80 registers this
+// kernel spills 176 bytes (28 at 96): 24 members of 26..205 by 130 cells, 40
+// steps, 14.35 ms with six CTAs, 13.69 with five (17.8 with the former kernel)
+template <typename T, int MODE, int WIDTH>
+__global__ void __launch_bounds__(32 * kRowWarps, (row_ctas<T, MODE>()) - 1)
     k_fire_ensemble_warp(const EnsembleArgs e) {
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     __shared__ StepArgs a;
@@ -172,7 +174,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, (row_ctas<T, NC ? ROW_NC : ROW
                 reinterpret_cast<int *>(&a)[q] = src[q];
             __syncthreads();
             sm.carve(dyn_smem, a.ky, a.sry, a.ncls);
-            RowStrip<T, NC ? ROW_NC : ROW_MULT, kRowWarps> strip(a, sm, dyn_smem);
+            RowStrip<T, MODE, kRowWarps, WIDTH> strip(a, sm, dyn_smem);
             strip.run(it.x0, it.y0, t);  // ends with a barrier
             const int stw = __reduce_or_sync(0xffffffffu, strip.st);
             if ((threadIdx.x & 31) == 0 && stw) atomicOr(a.status, stw);
@@ -233,6 +235,7 @@ struct fire_ensemble {
     cudaGraphExec_t graph = nullptr;
     bool capture_failed = false;
     int variant = FIRE_KERNEL_MARCH;  // member kernel: FIRE_KERNEL_MARCH or FIRE_KERNEL_WARP
+    bool even = true;  // every member's mesh has an even width
     bool nc = false;  // members carry per-node coefficients (a per-node fuel moisture)
     int g_nsteps = -1;
     double g_dt = 0;
@@ -272,6 +275,16 @@ void ens_release(fire_ensemble *e) {
     if (e->margs_host) cudaFreeHost(e->margs_host);
     if (e->run_host) cudaFreeHost(e->run_host);
     delete e;
+}
+
+// the warp form's kernel (FP32 only)
+const void *ens_warp_kernel(const fire_ensemble *e) {
+    const bool w = e->even;
+    if (e->nc)
+        return w ? (const void *)k_fire_ensemble_warp<float, ROW_NC, WIDTH_EVEN>
+                 : (const void *)k_fire_ensemble_warp<float, ROW_NC, WIDTH_ANY>;
+    return w ? (const void *)k_fire_ensemble_warp<float, ROW_MULT, WIDTH_EVEN>
+             : (const void *)k_fire_ensemble_warp<float, ROW_MULT, WIDTH_ANY>;
 }
 
 // work list and launch shape for the members' current kernel configuration
@@ -337,10 +350,7 @@ int ens_plan(fire_ensemble *e) {
     int threads;
     const bool f64 = e->prec == FIRE_FP64;
     if (e->variant == FIRE_KERNEL_WARP) {
-        fn = e->nc ? (f64 ? (const void *)k_fire_ensemble_warp<double, true>
-                          : (const void *)k_fire_ensemble_warp<float, true>)
-                   : (f64 ? (const void *)k_fire_ensemble_warp<double, false>
-                          : (const void *)k_fire_ensemble_warp<float, false>);
+        fn = ens_warp_kernel(e);
         threads = 32 * kRowWarps;
     } else {
         fn = e->nc ? (f64 ? (const void *)k_fire_ensemble<double, true>
@@ -353,10 +363,11 @@ int ens_plan(fire_ensemble *e) {
         // the limit is a property of the kernel function on a device, shared by
         // all ensembles there
         static std::mutex mu;
-        static size_t current[kMaxDevices][8] = {};
+        static size_t current[kMaxDevices][16] = {};
         std::lock_guard<std::mutex> lock(mu);
         const int dev = attr_device();
-        const int form = (f64 ? 1 : 0) + (e->variant == FIRE_KERNEL_WARP ? 2 : 0) + (e->nc ? 4 : 0);
+        const int form = (f64 ? 1 : 0) + (e->variant == FIRE_KERNEL_WARP ? 2 : 0) + (e->nc ? 4 : 0) +
+                         (e->even ? 8 : 0);
         if (dev < 0 || smem > current[dev][form]) {
             ENS_CHECK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             if (dev >= 0) current[dev][form] = smem;
@@ -396,11 +407,8 @@ cudaError_t ens_launch(fire_ensemble *e, double dt, cudaStream_t s) {
     cfg.numAttrs = 1;
     const bool f64 = e->prec == FIRE_FP64;
     if (e->variant == FIRE_KERNEL_WARP) {
-        if (e->nc)
-            return f64 ? cudaLaunchKernelEx(&cfg, k_fire_ensemble_warp<double, true>, ea)
-                       : cudaLaunchKernelEx(&cfg, k_fire_ensemble_warp<float, true>, ea);
-        return f64 ? cudaLaunchKernelEx(&cfg, k_fire_ensemble_warp<double, false>, ea)
-                   : cudaLaunchKernelEx(&cfg, k_fire_ensemble_warp<float, false>, ea);
+        void *args[] = {&ea};
+        return cudaLaunchKernelExC(&cfg, ens_warp_kernel(e), args);
     }
     if (e->nc)
         return f64 ? cudaLaunchKernelEx(&cfg, k_fire_ensemble<double, true>, ea)
@@ -457,6 +465,7 @@ int fire_ensemble_create(fire_ensemble **out, int n_members, const fire_member_d
             int prc, variant, nx, ny, srx, sry, kx, ky, ncls, cur;
             double t;
             ctx_info(c, &prc, &variant, &nx, &ny, &srx, &sry, &kx, &ky, &ncls, &cur, &t);
+            e->even = e->even && (nx & 1) == 0;
             warp = warp && srx <= kWarpMaxColumns / 2 && (long long)nx * ny <= kWarpMaxNodes;
         }
         e->variant = warp ? FIRE_KERNEL_WARP : FIRE_KERNEL_MARCH;

@@ -216,8 +216,12 @@ enum { ROW_PLAIN = 0, ROW_MULT = 1, ROW_NC = 2 };
 
 // how a strip lies in the mesh: any; or inside, on a mesh of even or odd width
 enum { EDGE = 0, PAIR = 1, SINGLE = 2 };
+// the mesh widths a kernel is compiled for: even, odd, or either (an ensemble
+// of both).  (With the bodies of both widths in one kernel the even one's
+// registers came out worse: 8200^2 nodes 663 -> 740 us.)
+enum { WIDTH_EVEN = 0, WIDTH_ODD = 1, WIDTH_ANY = 2 };
 
-template <typename T, int MODE, int NW>
+template <typename T, int MODE, int NW, int WIDTH>
 struct RowStrip {
     using V = typename PairT<T>::t;
     using S = RowSmem<T, NW>;
@@ -462,11 +466,13 @@ struct RowStrip {
                            y0 + La <= ny - band;
         if (inner) {
             if constexpr (sizeof(T) == 4) {
-                if ((nx & 1) == 0) loop<PAIR>();
+                if constexpr (WIDTH == WIDTH_EVEN) loop<PAIR>();
+                else if constexpr (WIDTH == WIDTH_ODD) loop<SINGLE>();
+                else if ((nx & 1) == 0) loop<PAIR>();
                 else loop<SINGLE>();
             }
         } else {
-            vec = (nx & 1) == 0;
+            vec = WIDTH == WIDTH_EVEN || (WIDTH == WIDTH_ANY && (nx & 1) == 0);
             inA = xa >= 0 && xa < nx;
             inB = xa + 1 >= 0 && xa + 1 < nx;
             pst = vec && outA && outB;
@@ -887,7 +893,7 @@ struct RowStrip {
 // most that many (the wind table of a CTA); the results do not depend on it
 inline int row_strip_bands(int ky, int sry) { return ky < kRowMaxBands ? ky : kRowMaxBands; }
 
-template <typename T, int MODE>
+template <typename T, int MODE, int WIDTH>
 __global__ void __launch_bounds__(32 * kRowWarps, (row_ctas<T, MODE>())) k_fire_warp(const StepArgs a) {
     extern __shared__ __align__(16) unsigned char row_smem[];
     constexpr int NW = kRowWarps;
@@ -895,7 +901,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, (row_ctas<T, MODE>())) k_fire_
     sm.carve(row_smem, a.ky, a.sry, a.ncls);
     const double tstart = *a.t_in;
     if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0) *a.t_out = tstart + a.dt;
-    RowStrip<T, MODE, NW> s(a, sm, row_smem);
+    RowStrip<T, MODE, NW, WIDTH> s(a, sm, row_smem);
     s.run(blockIdx.x * a.kx * a.srx, blockIdx.y * a.ky * a.sry, tstart);
     const int stw = __reduce_or_sync(0xffffffffu, s.st);
     if ((threadIdx.x & 31) == 0 && stw) atomicOr(a.status, stw);
@@ -915,7 +921,9 @@ cudaError_t prepare_warp_kernel(size_t smem_bytes) {
     const int dev = attr_device();
     if (dev >= 0 && smem_bytes <= current[dev]) return cudaSuccess;
     cudaError_t e = cudaSuccess;
-    for (auto k : {k_fire_warp<T, ROW_PLAIN>, k_fire_warp<T, ROW_MULT>, k_fire_warp<T, ROW_NC>})
+    for (auto k : {k_fire_warp<T, ROW_PLAIN, WIDTH_EVEN>, k_fire_warp<T, ROW_MULT, WIDTH_EVEN>,
+                   k_fire_warp<T, ROW_NC, WIDTH_EVEN>, k_fire_warp<T, ROW_PLAIN, WIDTH_ODD>,
+                   k_fire_warp<T, ROW_MULT, WIDTH_ODD>, k_fire_warp<T, ROW_NC, WIDTH_ODD>})
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
     if (e == cudaSuccess && dev >= 0) current[dev] = smem_bytes;
@@ -935,9 +943,10 @@ cudaError_t launch_warp(const StepArgs &args, cudaStream_t s) {
     const size_t smem = warp_smem_bytes<T>(a.ky, a.sry, a.ncls);
     cudaError_t e = prepare_warp_kernel<T>(smem);
     if (e != cudaSuccess) return e;
-    const auto k = a.nco[0] ? k_fire_warp<T, ROW_NC>
-                   : a.mult ? k_fire_warp<T, ROW_MULT>
-                            : k_fire_warp<T, ROW_PLAIN>;
+    const bool even = (a.nx & 1) == 0;
+    const auto k = a.nco[0] ? (even ? k_fire_warp<T, ROW_NC, WIDTH_EVEN> : k_fire_warp<T, ROW_NC, WIDTH_ODD>)
+                   : a.mult ? (even ? k_fire_warp<T, ROW_MULT, WIDTH_EVEN> : k_fire_warp<T, ROW_MULT, WIDTH_ODD>)
+                            : (even ? k_fire_warp<T, ROW_PLAIN, WIDTH_EVEN> : k_fire_warp<T, ROW_PLAIN, WIDTH_ODD>);
     k<<<grid, 32 * kRowWarps, smem, s>>>(a);
     return cudaGetLastError();
 }
