@@ -50,6 +50,7 @@ namespace wf {
 
 int ctx_step_args(fire_ctx *c, int parity, const void *u, const void *v, double dt, double *hs,
                   double *hl, StepArgs &a);
+int ctx_launch_variant(const fire_ctx *c);
 int ctx_info(const fire_ctx *c, int *prec, int *variant, int *nx, int *ny, int *srx, int *sry,
              int *kx, int *ky, int *ncls, int *cur, double *t);
 int ctx_advance(fire_ctx *c, int nsteps, double dt);
@@ -1321,6 +1322,7 @@ int run_adjoint(fire_ctx *c, int nsteps, double dt, const void *u, const void *v
     int prec, variant, nx, ny, srx, sry, kx, ky, ncls, cur;
     double t0;
     ctx_info(c, &prec, &variant, &nx, &ny, &srx, &sry, &kx, &ky, &ncls, &cur, &t0);
+    variant = ctx_launch_variant(c);
     const cudaStream_t st = ctx_stream(c);
     const size_t n = (size_t)nx * ny, E = sizeof(T);
     const bool grads = g_mult || g_moist || g_u || g_v;

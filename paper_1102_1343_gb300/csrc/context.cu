@@ -50,7 +50,7 @@ struct fire_ctx {
 
     int variant = FIRE_KERNEL_MARCH;
     int kx = 0, ky = 0;
-    int launch_ky = 0;  // rows of a CTA of the default warp strips (0: ky)
+    DefaultShape launch{FIRE_KERNEL_MARCH, 0, 0};  // kernel and shape of its launches (launch_shape)
     int scheme = 0;  // fuel fraction: 0 subcell scheme, 1 exact for linear data (tiles)
     size_t smem = 0;
     size_t smem_max = 0;
@@ -65,7 +65,7 @@ struct fire_ctx {
     const void *g_u = nullptr, *g_v = nullptr;
     double g_dt = 0;
     double *g_hs = nullptr, *g_hl = nullptr;
-    int g_kx = 0, g_ky = 0, g_launch_ky = 0, g_variant = -1;
+    DefaultShape g_launch{-1, 0, 0};
 
     // workspace of fire_adjoint (grown on demand, freed with the context)
     void *ws = nullptr;
@@ -87,7 +87,7 @@ struct fire_ctx {
     bool adaptive = false;
     bool ad_dense = false;                       // the dense variant is chosen
     int ad_kx = 0, ad_ky = 0, ad_dense_ky = 0;   // the two shapes
-    bool ad_launch = false;                      // CTAs of warp_launch_rows (fire_init's default)
+    bool ad_launch = false;                      // launches by launch_shape (fire_init's default)
     unsigned long long *ad_count_dev = nullptr;  // nodes with psi <= 0
     unsigned long long *ad_count_host = nullptr; // page-locked copy of it
     cudaEvent_t ad_ready = nullptr;              // that copy has landed
@@ -222,8 +222,8 @@ int step_kernel_args(fire_ctx *c, const void *u, const void *v, double dt, doubl
     a.nya = c->g.ny_atm;
     a.srx = c->g.sr_x;
     a.sry = c->g.sr_y;
-    a.kx = c->kx;
-    a.ky = c->launch_ky ? c->launch_ky : c->ky;
+    a.kx = c->launch.kx;
+    a.ky = c->launch.ky;
     a.band = c->g.boundary_band;
     a.dx = c->dx;
     a.dy = c->dy;
@@ -233,13 +233,13 @@ int step_kernel_args(fire_ctx *c, const void *u, const void *v, double dt, doubl
 }
 
 cudaError_t launch_variant(const fire_ctx *c, const StepArgs &a, cudaStream_t s) {
-    if (c->variant == FIRE_KERNEL_MARCH)
+    if (c->launch.variant == FIRE_KERNEL_MARCH)
         return c->prec == FIRE_FP64 ? launch_march<double>(a, s) : launch_march<float>(a, s);
-    if (c->variant == FIRE_KERNEL_WARP)
+    if (c->launch.variant == FIRE_KERNEL_WARP)
         return c->prec == FIRE_FP64 ? launch_warp<double>(a, s) : launch_warp<float>(a, s);
-    if (c->variant == FIRE_KERNEL_WARP4)
+    if (c->launch.variant == FIRE_KERNEL_WARP4)
         return c->prec == FIRE_FP32 ? launch_warp4(a, s) : cudaErrorInvalidValue;
-    if (c->variant == FIRE_KERNEL_WARP_DENSE)
+    if (c->launch.variant == FIRE_KERNEL_WARP_DENSE)
         return c->prec == FIRE_FP32 ? launch_warp<float>(a, s) : cudaErrorInvalidValue;
     return c->prec == FIRE_FP64 ? launch_step<double>(a, s) : launch_step<float>(a, s);
 }
@@ -351,15 +351,15 @@ int configure_kernel(fire_ctx *c, int variant, int kx, int ky) {
     c->variant = variant;
     c->kx = kx;
     c->ky = ky;
-    c->launch_ky = 0;
+    c->launch = DefaultShape{variant, kx, ky};
     c->smem = sm;
     return FIRE_OK;
 }
 
-// the rows that a CTA takes of the default warp strips
-void default_launch_rows(fire_ctx *c) {
-    if (c->variant == FIRE_KERNEL_WARP || c->variant == FIRE_KERNEL_WARP_DENSE)
-        c->launch_ky = warp_launch_rows(c->nx, c->ny, c->kx * c->g.sr_x, c->g.sr_y, c->n_sm);
+// what launches take in place of the default shape
+void default_launch(fire_ctx *c) {
+    c->launch = launch_shape(c->prec == FIRE_FP64, DefaultShape{c->variant, c->kx, c->ky}, c->g.nx_atm,
+                             c->g.ny_atm, c->g.sr_x, c->g.sr_y, c->ncls, c->n_sm, c->smem_max);
 }
 
 // marching strips of up to 248 columns (an even number) x ~60 rows
@@ -393,7 +393,7 @@ int default_kernel(fire_ctx *c) {
     const DefaultShape d = default_shape(c->prec == FIRE_FP64, c->g.nx_atm, c->g.ny_atm,
                                          c->g.sr_x, c->g.sr_y, c->n_sm);
     if (configure_kernel(c, d.variant, d.kx, d.ky) == FIRE_OK) {
-        default_launch_rows(c);
+        default_launch(c);
         return FIRE_OK;
     }
     // a strip shape whose shared memory does not fit: 2-D tiles, halved until
@@ -444,7 +444,7 @@ int adaptive_decide(fire_ctx *c, unsigned long long count) {
                                    dense ? c->ad_dense_ky : c->ad_ky);
     if (r != FIRE_OK) return r;
     c->ad_dense = dense;
-    if (c->ad_launch) default_launch_rows(c);
+    if (c->ad_launch) default_launch(c);
     return FIRE_OK;
 }
 
@@ -502,7 +502,7 @@ void adaptive_setup(fire_ctx *c) {
     c->ad_dense = false;
     c->ad_kx = c->kx;
     c->ad_ky = c->ky;
-    c->ad_launch = c->launch_ky != 0;
+    c->ad_launch = c->launch != DefaultShape{c->variant, c->kx, c->ky};
     const int short_rows = 60 / c->g.sr_y;
     c->ad_dense_ky = c->ky < short_rows ? c->ky : (short_rows < 1 ? 1 : short_rows);
     c->ad_steps = kAdaptEvery;  // count before the first step
@@ -595,8 +595,8 @@ DefaultShape default_shape(bool fp64, int nx_atm, int ny_atm, int srx, int sry, 
     return {FIRE_KERNEL_TILE, kx, ky};
 }
 
-int warp_launch_rows(int nx, int ny, int W, int sry, int n_sm) {
-    const long strips = cdiv_l(nx, W), slots = (long)n_sm * kRowCtasPerSmF32;
+int warp_launch_rows(bool fp64, int nx, int ny, int W, int sry, int n_sm) {
+    const long strips = cdiv_l(nx, W), slots = (long)n_sm * (fp64 ? kRowCtasPerSmF64 : kRowCtasPerSmF32);
     int best = 1;
     double least = 0;
     for (int ky = 1; ky <= kRowMaxBands && (ky == 1 || (ky - 1) * (long)sry < ny) && (ky == 1 || ky * (long)sry <= kWarpMaxRows); ++ky) {
@@ -609,6 +609,52 @@ int warp_launch_rows(int nx, int ny, int W, int sry, int n_sm) {
     }
     return best;
 }
+
+DefaultShape launch_shape(bool fp64, const DefaultShape &d, int nx_atm, int ny_atm, int srx, int sry,
+                          int ncls, int n_sm, size_t smem_max) {
+    const long long nx = (long long)nx_atm * srx, ny = (long long)ny_atm * sry;
+    DefaultShape r = d;
+    if (d.variant == FIRE_KERNEL_WARP || d.variant == FIRE_KERNEL_WARP_DENSE) {
+        r.ky = warp_launch_rows(fp64, (int)nx, (int)ny, d.kx * srx, sry, n_sm);
+    } else if (d.variant == FIRE_KERNEL_MARCH && fp64) {
+        int kx = kWarpMaxColumns / srx;
+        if (kx > nx_atm) kx = nx_atm;
+        if ((kx * srx) & 1) kx = kx > 1 ? kx - 1 : 2;
+        const int W = kx * srx;
+        if (kx < 1 || W > kWarpMaxColumns || (W < kRowMinColumns && W < nx) || sry > kWarpMaxRows ||
+            nx * ny > kWarpMaxNodes)
+            return d;
+        const int ky = warp_launch_rows(true, (int)nx, (int)ny, W, sry, n_sm);
+        if (warp_smem_bytes<double>(ky, sry, ncls) > smem_max) return d;
+        r = DefaultShape{FIRE_KERNEL_WARP, kx, ky};
+    } else if (d.variant == FIRE_KERNEL_TILE) {
+        // a wave of resident CTAs takes a time of its own (the chain of stages)
+        // and one of the nodes that its tiles compute in the three stages
+        const long slots = (long)n_sm * (fp64 ? kTileCtasPerSmF64 : kTileCtasPerSmF32);
+        const double own = fp64 ? 140 : 3000;
+        static const int step[] = {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48};
+        double least = 0;
+        for (int kx : step)
+            for (int ky : step) {
+                const long TX = (long)kx * srx, TY = (long)ky * sry;
+                if ((kx > 1 && kx > nx_atm) || (ky > 1 && ky > ny_atm) || TX > 48 || TY > 48) break;
+                const size_t sm = fp64 ? step_table_bytes<double>(kx, ky, srx, sry, ncls)
+                                       : step_table_bytes<float>(kx, ky, srx, sry, ncls);
+                if (!sm) break;
+                const long waves = cdiv_l(cdiv_l(nx_atm, kx) * cdiv_l(ny_atm, ky), slots);
+                const double t = waves * (own + (TX + 4) * (TY + 4) + (TX + 2) * (TY + 2) + TX * TY);
+                if (least == 0 || t < least) {
+                    least = t;
+                    r = DefaultShape{FIRE_KERNEL_TILE, kx, ky};
+                }
+            }
+    }
+    return r;
+}
+
+// the kernel that the context's launches take (its shape stands in the step
+// arguments)
+int ctx_launch_variant(const fire_ctx *c) { return c->launch.variant; }
 
 int ctx_step_args(fire_ctx *c, int parity, const void *u, const void *v, double dt, double *hs,
                   double *hl, StepArgs &a) {
@@ -953,8 +999,7 @@ int fire_run(fire_ctx *c, int nsteps, double dt, const void *u, const void *v, d
         if (ra) return ra;
         c->ad_steps += 2;
         if (!c->graph || c->g_u != u || c->g_v != v || c->g_dt != dt || c->g_hs != hs ||
-            c->g_hl != hl || c->g_kx != c->kx || c->g_ky != c->ky ||
-            c->g_launch_ky != c->launch_ky || c->g_variant != c->variant) {
+            c->g_hl != hl || c->g_launch != c->launch) {
             if (c->graph) {
                 WF_CHECK(cudaStreamSynchronize(c->stream));  // the old graph may be in flight
                 cudaGraphExecDestroy(c->graph);
@@ -988,10 +1033,7 @@ int fire_run(fire_ctx *c, int nsteps, double dt, const void *u, const void *v, d
             c->g_dt = dt;
             c->g_hs = hs;
             c->g_hl = hl;
-            c->g_kx = c->kx;
-            c->g_ky = c->ky;
-            c->g_launch_ky = c->launch_ky;
-            c->g_variant = c->variant;
+            c->g_launch = c->launch;
         }
         WF_CHECK(cudaGraphLaunch(c->graph, c->stream));
         c->t = c->t + dt;

@@ -105,6 +105,11 @@ struct IgniteArgs {
 template <typename T>
 size_t step_smem_bytes(int kx, int ky, int srx, int sry, int ncls);
 
+// shared memory of the tile kernel's form with wind tables, 0: a tile too
+// large for it
+template <typename T>
+size_t step_table_bytes(int kx, int ky, int srx, int sry, int ncls);
+
 template <typename T>
 cudaError_t launch_step(const StepArgs &a, cudaStream_t s);
 
@@ -144,6 +149,9 @@ cudaError_t launch_warp4(const StepArgs &a, cudaStream_t s);
 
 constexpr int kRowWarps = 4;         // warps of a CTA of the warp kernel, one row each at a time
 constexpr int kRowCtasPerSmF32 = 6;  // its resident CTAs per SM that the registers allow
+constexpr int kRowCtasPerSmF64 = 2;
+constexpr int kTileCtasPerSmF32 = 4;  // and of the tile kernel
+constexpr int kTileCtasPerSmF64 = 2;
 constexpr int kRowMaxBands = 16;     // atmospheric rows of one CTA of it at most
 constexpr int kWarpStrips = 4;       // warps (strips) per CTA of the four-column warp kernel
 constexpr int kWarpMaxColumns = 60;  // output columns of one warp strip (even)
@@ -170,6 +178,10 @@ constexpr int kMarchCtasPerSmF64 = 2;
 // checks the shape's shared memory and halves tiles that do not fit.
 struct DefaultShape {
     int variant, kx, ky;
+    bool operator==(const DefaultShape &o) const {
+        return variant == o.variant && kx == o.kx && ky == o.ky;
+    }
+    bool operator!=(const DefaultShape &o) const { return !(*this == o); }
 };
 DefaultShape default_shape(bool fp64, int nx_atm, int ny_atm, int srx, int sry, int n_sm);
 
@@ -181,7 +193,26 @@ DefaultShape default_shape(bool fp64, int nx_atm, int ny_atm, int srx, int sry, 
 // the measured best: 2000^2 nodes 30 rows (10: 100 us, 30: 64, 60: 69, 160:
 // 100), 1000^2 20 rows (10: 32 us, 20: 27, 30: 30), 510^2 10 rows (10: 14.5,
 // 20: 20).
-int warp_launch_rows(int nx, int ny, int W, int sry, int n_sm);
+// FP64 (two CTAs per SM): 2000^2 nodes 40 rows (10: 1613 us, 20: 1376, 30: 1327,
+// 40: 1309, 60: 1350), 1000^2 20 rows (10: 449, 20: 423, 40: 490), 510^2 10
+// rows (10: 195, 20: 185, 40: 248).
+int warp_launch_rows(bool fp64, int nx, int ny, int W, int sry, int n_sm);
+
+// What launches take in place of the default shape d (fire_init,
+// fire_step_noalloc; d is what fire_get_kernel reports, and the results are
+// the same bits):
+// - warp strips: the rows of warp_launch_rows;
+// - FP64 marching strips: the warp kernel's strips, where they are at least
+//   kRowMinColumns wide (below, its lanes that hang over cost more than it
+//   gains: the time goes with 64 over the width).  us per step, marching and
+//   now: 2000^2 nodes 1611 and 1309, 1000^2 565 and 423, 510^2 322 and 185;
+// - tiles: of several cells, with tables, where they come out in fewer waves
+//   of resident CTAs.  FP64 370x290: 1x1 119 us, 1x2 98, 2x2 94; 200^2: 1x1 64,
+//   1x2 49, 2x2 65; 100^2: 1x1 30, 1x2 46.  FP32 370x290: 1x1 21.6, 2x1 14.4,
+//   2x2 13.5; 200^2: 1x1 11.4, 2x2 12.4.
+DefaultShape launch_shape(bool fp64, const DefaultShape &d, int nx_atm, int ny_atm, int srx, int sry,
+                          int ncls, int n_sm, size_t smem_max);
+constexpr int kRowMinColumns = 50;
 
 cudaError_t launch_coefficients(const fire_fuel_class *classes_dev, int n, double *coef_dev,
                                 cudaStream_t s);

@@ -165,12 +165,14 @@ extern "C" int fire_step_noalloc(const fire_grid_desc *grid, const fire_fuel_cla
         cudaDeviceGetAttribute(&smo, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return FIRE_ERR_CUDA;
-    const DefaultShape d = default_shape(fp64, g.nx_atm, g.ny_atm, g.sr_x, g.sr_y, n_sm);
+    const DefaultShape d0 = default_shape(fp64, g.nx_atm, g.ny_atm, g.sr_x, g.sr_y, n_sm);
+    const DefaultShape d =
+        launch_shape(fp64, d0, g.nx_atm, g.ny_atm, g.sr_x, g.sr_y, n_classes, n_sm, (size_t)smo);
     cudaError_t e = cudaErrorInvalidValue;
     if (d.variant == FIRE_KERNEL_WARP && (long long)d.ky * g.sr_y <= kWarpMaxRows) {
         a.kx = d.kx;
-        a.ky = warp_launch_rows(a.nx, a.ny, d.kx * g.sr_x, g.sr_y, n_sm);
-        e = launch_warp<float>(a, st);
+        a.ky = d.ky;
+        e = fp64 ? launch_warp<double>(a, st) : launch_warp<float>(a, st);
         return e == cudaSuccess ? FIRE_OK : FIRE_ERR_CUDA;
     }
     if (d.variant == FIRE_KERNEL_MARCH) {

@@ -149,7 +149,8 @@ __host__ __device__ inline size_t tile_wind_elems(int TX, int TY, int ky) {
 // in FP64 53.7 and 30.0.
 // ---------------------------------------------------------------------------
 template <typename T, bool TAB>
-__global__ void __launch_bounds__(kThreads) k_fire_step(const StepArgs a) {
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 : kTileCtasPerSmF32)
+    k_fire_step(const StepArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_status;
     const int tid = threadIdx.x;
@@ -622,7 +623,7 @@ size_t step_smem_bytes(int kx, int ky, int srx, int sry, int ncls) {
 // CTA: past a quarter of the SM's shared memory the wind is interpolated per
 // node instead
 template <typename T>
-static size_t tile_tab_bytes(int kx, int ky, int srx, int sry, int ncls) {
+size_t step_table_bytes(int kx, int ky, int srx, int sry, int ncls) {
     const size_t n = tile_elems<T>(kx * srx, ky * sry, ncls) + tile_wind_elems<T>(kx * srx, ky * sry, ky);
     return n * sizeof(T) <= kTileTabBytes ? n * sizeof(T) : 0;
 }
@@ -650,7 +651,7 @@ cudaError_t launch_step(const StepArgs &a, cudaStream_t s) {
     const int TX = a.kx * a.srx, TY = a.ky * a.sry;
     dim3 grid((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY);
     const size_t smem = step_smem_bytes<T>(a.kx, a.ky, a.srx, a.sry, a.ncls);
-    const size_t tab = tile_tab_bytes<T>(a.kx, a.ky, a.srx, a.sry, a.ncls);
+    const size_t tab = step_table_bytes<T>(a.kx, a.ky, a.srx, a.sry, a.ncls);
     cudaError_t e = prepare_step_kernel<T>(smem);
     if (e != cudaSuccess) return e;
     if (tab)
@@ -681,6 +682,7 @@ cudaError_t launch_fill(void *psi, double *tign, void *frac, size_t n, double ps
 
 #define WF_INSTANTIATE(T)                                                                     \
     template size_t step_smem_bytes<T>(int, int, int, int, int);                              \
+    template size_t step_table_bytes<T>(int, int, int, int, int);                             \
     template cudaError_t prepare_step_kernel<T>(size_t);                                      \
     template cudaError_t launch_step<T>(const StepArgs &, cudaStream_t);                      \
     template cudaError_t launch_ignite<T>(const IgniteArgs &, cudaStream_t);                  \

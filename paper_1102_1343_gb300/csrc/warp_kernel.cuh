@@ -64,7 +64,7 @@ struct WRow {  // y-interpolation of the wind for one fire row
 // need 96
 template <typename T, int MODE>
 constexpr int row_ctas() {
-    return sizeof(T) == 8 ? 1 : MODE == 2 ? 5 : kRowCtasPerSmF32;
+    return sizeof(T) == 8 ? kRowCtasPerSmF64 : MODE == 2 ? 5 : kRowCtasPerSmF32;
 }
 
 // wind rows of a strip's table: its atmospheric rows and those around them
