@@ -331,7 +331,7 @@ int configure_kernel(fire_ctx *c, int variant, int kx, int ky) {
         sm = c->prec == FIRE_FP64 ? warp_smem_bytes<double>(kr, c->g.sr_y, c->ncls)
                                   : warp_smem_bytes<float>(kr, c->g.sr_y, c->ncls);
         if (sm > c->smem_max) return FIRE_ERR_ARG;
-        e = c->prec == FIRE_FP64 ? prepare_warp_kernel<double>(sm) : prepare_warp_kernel<float>(sm);
+        e = cudaSuccess;  // (launch_warp prepares the kernel it takes)
     } else if (variant == FIRE_KERNEL_WARP4) {
         const long long W = (long long)kx * c->g.sr_x, L = (long long)ky * c->g.sr_y;
         if (c->prec != FIRE_FP32 || W > kWarp4MaxColumns || L > kWarpMaxRows ||

@@ -59,7 +59,7 @@ struct StepArgs {
     const void *psi_in;
     void *psi_out;
     const void *F_in;
-    void *F_out;
+    void *F_out;  // null (warp and tile kernels): psi alone, without F, t_i and heat
     double *tign;
     const uint8_t *fuel;
     const void *dzdx, *dzdy, *mult;
@@ -136,9 +136,6 @@ constexpr int kMarchMaxColumns = 248;  // output columns of one marching strip (
 
 template <typename T>
 size_t warp_smem_bytes(int ky, int sry, int ncls);
-
-template <typename T>
-cudaError_t prepare_warp_kernel(size_t smem_bytes);
 
 template <typename T>
 cudaError_t launch_warp(const StepArgs &a, cudaStream_t s);

@@ -162,6 +162,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 :
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
     const int TXa = min(TX, nx - x0), TYa = min(TY, ny - y0);
     const int WR = TAB ? tile_wind_rows(a.ky) : 0;
+    // psi alone (states recomputed for the adjoint): no ignition times, no
+    // fuel fraction, no heat
+    const bool full = a.F_out != nullptr;
 
     T *lut = reinterpret_cast<T *>(smem_raw);
     T *P0 = lut + lut_slots<T>(a.ncls);
@@ -313,7 +316,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 :
         const T p0 = P0[(ly + 2) * BW3 + (lx + 2)];
         // t_i where the node burns already, read ahead of the arithmetic
         double ti = 0.0;
-        if (le0(p0)) ti = a.tign[g];
+        if (full && le0(p0)) ti = a.tign[g];
         int cls = fuel[g];
         cls = cls > ncm1 ? ncm1 : cls;
         const int c2 = (ly + 1) * BW2 + (lx + 1);
@@ -332,7 +335,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 :
         P2[l1] = pn;
         const bool own = lx >= 1 && lx <= TXa && ly >= 1 && ly <= TYa;
         T d = T(0);
-        if (le0(pn)) {
+        if (full && le0(pn)) {
             const bool cross = p0 > T(0) && pn <= T(0);
             if (cross || pn < T(0)) {
                 if (!le0(p0)) ti = a.tign[g];
@@ -351,6 +354,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 :
             const bool band = gx < a.band || gy < a.band || gx >= nx - a.band || gy >= ny - a.band;
             if (band && pn < T(0)) st |= ST_BOUNDARY;
         }
+    }
+    if (!full) {
+        if (st) atomicOr(a.status, st);
+        return;
     }
     __syncthreads();
     if (edge_tile) fill_ghosts_pd<T>(P2, Dl, BW1, BH1, x0 - 1, y0 - 1, nx, ny, tid);

@@ -221,7 +221,9 @@ enum { EDGE = 0, PAIR = 1, SINGLE = 2 };
 // registers came out worse: 8200^2 nodes 663 -> 740 us.)
 enum { WIDTH_EVEN = 0, WIDTH_ODD = 1, WIDTH_ANY = 2 };
 
-template <typename T, int MODE, int NW, int WIDTH>
+// FULL: false for a step of psi alone (no F_out: states recomputed for the
+// adjoint), without stages 3 to 5 and the ignition times
+template <typename T, int MODE, int NW, int WIDTH, bool FULL = true>
 struct RowStrip {
     using V = typename PairT<T>::t;
     using S = RowSmem<T, NW>;
@@ -519,7 +521,8 @@ struct RowStrip {
         int bdone = 0;     // bands ended by stage 4 before this iteration
         int bavg = 0;      // bands averaged by stage 5
         unsigned f1 = 0;   // flags of iteration i - 2
-        int left = (La + 3) / NW + 5;  // iterations left
+        // iterations left (psi alone: until stage 2 has taken row La - 1)
+        int left = FULL ? (La + 3) / NW + 5 : (La + 3 + NW - 1) / NW + 1;
         unsigned n1 = w * kRow;        // ring offset of stage 1's row
         unsigned aw = smem_addr(sm.rows + w);  // wind weights of stage 1's row
         // bytes w + 2 .. w + 4 of two iterations' flags: rows k3 - 1 .. k3 + 1
@@ -527,12 +530,12 @@ struct RowStrip {
         unsigned af = sflag, ad = S::DF;  // flags, dF rows of iteration i (two sets in turn)
 #pragma unroll 1
         for (; left > 0; --left) {
-            const unsigned f0 = lds_u32(af ^ 4);  // flags of iteration i - 1
+            const unsigned f0 = FULL ? lds_u32(af ^ 4) : 0u;  // flags of iteration i - 1
             int flag = 0;
             const unsigned n2 = (n1 - (NW + 1) * kRow) & (kN - 1);
             // ---- stage 3 on row k3
             const int k3 = k - 2 * NW - 2;
-            if ((unsigned)k3 < (unsigned)La) {
+            if (FULL && (unsigned)k3 < (unsigned)La) {
                 // flags of rows k3 - 1, k3, k3 + 1: warps w - 2, w - 1, w of
                 // iteration i - 1, counted on from those of i - 2
                 const unsigned burn = __byte_perm(f1, f0, sel);
@@ -544,10 +547,10 @@ struct RowStrip {
             // the registers whose last use is just behind, so that nothing
             // waits for it before the next iteration)
             const int k2 = k - NW - 1;
-            if ((unsigned)(k2 + 1) <= (unsigned)(La + 1)) {
+            if (FULL ? (unsigned)(k2 + 1) <= (unsigned)(La + 1) : (unsigned)k2 < (unsigned)La) {
                 if (FORM != EDGE || (y0 + k2 >= 0 && y0 + k2 < ny))
                     flag |= stage2<FORM>(y0 + k2, o1 - (NW + 1) * nx, n2, e2) ? 1 : 0;
-                Fn = ld<FORM>(a.F_in, y0 + k2 - 1, o1 - (NW + 2) * nx);
+                if (FULL) Fn = ld<FORM>(a.F_in, y0 + k2 - 1, o1 - (NW + 2) * nx);
             }
             // ---- stage 1 on row k; loads of its next row
             if (k <= La + 1) {
@@ -575,32 +578,34 @@ struct RowStrip {
                 }
                 if (k + NW <= La + 1) load1(y0 + k + NW, o1 + NW * nx);
             }
-            f1 = f0;
-            if (lane == 0) sts_u8(af + w, flag);
-            // ---- stage 5: averages of the bands ended in iteration i - 1
-            for (; bavg < bdone; ++bavg) average(bavg, (hotbits >> (bdone - 1 - bavg)) & 1u);
-            // ---- stage 4: heat of the rows stage 3 took in iteration i - 1
-            const int e4 = min(k3 - w, La);  // one past the last of them
-            if (e4 >= bend || (f0 & 0x02020202u)) {
-                const int rf = k3 - w - NW;  // the first (negative: none yet)
-                for (int r = max(d4, 0); r < e4; ++r) {
-                    if ((f0 >> (8 * (r - rf))) & 2u) {
-                        bhot = true;
-                        add_heat(y0 + r, (2 * S::DF + NW * kRow - ad) + (r - rf) * kRow, acc);
-                    }
-                    if (r + 1 == bend) {
-                        bend += sry;
-                        if (bhot) {
-                            sm.hw[(bdone % row_bands(NW, sry)) * 128 + (w < 2 ? 0 : 64) + (w & 1) * 32 + lane] = acc;
-                            acc = T(0);
+            if constexpr (FULL) {
+                f1 = f0;
+                if (lane == 0) sts_u8(af + w, flag);
+                // ---- stage 5: averages of the bands ended in iteration i - 1
+                for (; bavg < bdone; ++bavg) average(bavg, (hotbits >> (bdone - 1 - bavg)) & 1u);
+                // ---- stage 4: heat of the rows stage 3 took in iteration i - 1
+                const int e4 = min(k3 - w, La);  // one past the last of them
+                if (e4 >= bend || (f0 & 0x02020202u)) {
+                    const int rf = k3 - w - NW;  // the first (negative: none yet)
+                    for (int r = max(d4, 0); r < e4; ++r) {
+                        if ((f0 >> (8 * (r - rf))) & 2u) {
+                            bhot = true;
+                            add_heat(y0 + r, (2 * S::DF + NW * kRow - ad) + (r - rf) * kRow, acc);
                         }
-                        hotbits = (hotbits << 1) | (bhot ? 1u : 0u);
-                        bhot = false;
-                        ++bdone;
+                        if (r + 1 == bend) {
+                            bend += sry;
+                            if (bhot) {
+                                sm.hw[(bdone % row_bands(NW, sry)) * 128 + (w < 2 ? 0 : 64) + (w & 1) * 32 + lane] = acc;
+                                acc = T(0);
+                            }
+                            hotbits = (hotbits << 1) | (bhot ? 1u : 0u);
+                            bhot = false;
+                            ++bdone;
+                        }
                     }
                 }
+                d4 = e4;
             }
-            d4 = e4;
             k += NW;
             o1 += NW * nx;
             n1 = (n1 + NW * kRow) & (kN - 1);
@@ -659,7 +664,7 @@ struct RowStrip {
         // no new t_i in this step, so no other warp writes them)
         const bool fa = lane > 0 && (FORM != EDGE || inA), fb = lane < 31 && (FORM != EDGE || inB);
         double tiA = 0.0, tiB = 0.0;
-        if (__any_sync(0xffffffffu, min_val(P0.x, P0.y) <= T(0))) {
+        if (FULL && __any_sync(0xffffffffu, min_val(P0.x, P0.y) <= T(0))) {
             const int g = r * nx + xa;
             if (fa && P0.x <= T(0)) tiA = a.tign[WF_CHK(g, nx * ny, st)];
             if (fb && P0.y <= T(0)) tiB = a.tign[WF_CHK(g + 1, nx * ny, st)];
@@ -689,6 +694,7 @@ struct RowStrip {
             }
             store<FORM>(a.psi_out, r, off, N0);
         }
+        if constexpr (!FULL) return false;
         // ignition time and t - t_i, only where a node is burning
         const bool burn = __any_sync(0xffffffffu, min_val(N0.x, N0.y) <= T(0));
         if (burn) {
@@ -893,7 +899,7 @@ struct RowStrip {
 // most that many (the wind table of a CTA); the results do not depend on it
 inline int row_strip_bands(int ky, int sry) { return ky < kRowMaxBands ? ky : kRowMaxBands; }
 
-template <typename T, int MODE, int WIDTH>
+template <typename T, int MODE, int WIDTH, bool FULL>
 __global__ void __launch_bounds__(32 * kRowWarps, (row_ctas<T, MODE>())) k_fire_warp(const StepArgs a) {
     extern __shared__ __align__(16) unsigned char row_smem[];
     constexpr int NW = kRowWarps;
@@ -901,10 +907,28 @@ __global__ void __launch_bounds__(32 * kRowWarps, (row_ctas<T, MODE>())) k_fire_
     sm.carve(row_smem, a.ky, a.sry, a.ncls);
     const double tstart = *a.t_in;
     if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0) *a.t_out = tstart + a.dt;
-    RowStrip<T, MODE, NW, WIDTH> s(a, sm, row_smem);
+    RowStrip<T, MODE, NW, WIDTH, FULL> s(a, sm, row_smem);
     s.run(blockIdx.x * a.kx * a.srx, blockIdx.y * a.ky * a.sry, tstart);
     const int stw = __reduce_or_sync(0xffffffffu, s.st);
     if ((threadIdx.x & 31) == 0 && stw) atomicOr(a.status, stw);
+}
+
+// the kernel of a mode, a parity of the mesh width, and the full step or psi
+// alone
+using RowKernel = void (*)(const StepArgs);
+template <typename T, bool FULL>
+RowKernel row_kernel_of(int mode, bool even) {
+    switch (mode) {
+        case ROW_NC: return even ? k_fire_warp<T, ROW_NC, WIDTH_EVEN, FULL> : k_fire_warp<T, ROW_NC, WIDTH_ODD, FULL>;
+        case ROW_MULT:
+            return even ? k_fire_warp<T, ROW_MULT, WIDTH_EVEN, FULL> : k_fire_warp<T, ROW_MULT, WIDTH_ODD, FULL>;
+        default:
+            return even ? k_fire_warp<T, ROW_PLAIN, WIDTH_EVEN, FULL> : k_fire_warp<T, ROW_PLAIN, WIDTH_ODD, FULL>;
+    }
+}
+template <typename T>
+RowKernel row_kernel(int mode, bool even, bool full) {
+    return full ? row_kernel_of<T, true>(mode, even) : row_kernel_of<T, false>(mode, even);
 }
 
 template <typename T>
@@ -912,21 +936,19 @@ size_t warp_smem_bytes(int ky, int sry, int ncls) {
     return RowSmem<T, kRowWarps>::bytes(ky, sry, ncls);
 }
 
-// raised monotonically: the limit is shared by every context in the process
+// raised monotonically, kernel by kernel as each is first launched (setting
+// it loads the kernel, a third of a millisecond): the limit is shared by every
+// context in the process
 template <typename T>
-cudaError_t prepare_warp_kernel(size_t smem_bytes) {
+cudaError_t prepare_row_kernel(int mode, bool even, bool full, size_t smem_bytes) {
     static std::mutex mu;
-    static size_t current[kMaxDevices] = {};  // per device (the attribute is)
+    static size_t current[kMaxDevices][12] = {};  // per device (the attribute is)
     std::lock_guard<std::mutex> lock(mu);
-    const int dev = attr_device();
-    if (dev >= 0 && smem_bytes <= current[dev]) return cudaSuccess;
-    cudaError_t e = cudaSuccess;
-    for (auto k : {k_fire_warp<T, ROW_PLAIN, WIDTH_EVEN>, k_fire_warp<T, ROW_MULT, WIDTH_EVEN>,
-                   k_fire_warp<T, ROW_NC, WIDTH_EVEN>, k_fire_warp<T, ROW_PLAIN, WIDTH_ODD>,
-                   k_fire_warp<T, ROW_MULT, WIDTH_ODD>, k_fire_warp<T, ROW_NC, WIDTH_ODD>})
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
-    if (e == cudaSuccess && dev >= 0) current[dev] = smem_bytes;
+    const int dev = attr_device(), k = mode * 4 + (even ? 2 : 0) + (full ? 1 : 0);
+    if (dev >= 0 && smem_bytes <= current[dev][k]) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(row_kernel<T>(mode, even, full),
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+    if (e == cudaSuccess && dev >= 0) current[dev][k] = smem_bytes;
     return e;
 }
 
@@ -941,19 +963,16 @@ cudaError_t launch_warp(const StepArgs &args, cudaStream_t s) {
     const int L = a.ky * a.sry;
     dim3 grid((a.nx + W - 1) / W, (a.ny + L - 1) / L);
     const size_t smem = warp_smem_bytes<T>(a.ky, a.sry, a.ncls);
-    cudaError_t e = prepare_warp_kernel<T>(smem);
+    const int mode = a.nco[0] ? ROW_NC : a.mult ? ROW_MULT : ROW_PLAIN;
+    const bool even = (a.nx & 1) == 0, full = a.F_out != nullptr;
+    const cudaError_t e = prepare_row_kernel<T>(mode, even, full, smem);
     if (e != cudaSuccess) return e;
-    const bool even = (a.nx & 1) == 0;
-    const auto k = a.nco[0] ? (even ? k_fire_warp<T, ROW_NC, WIDTH_EVEN> : k_fire_warp<T, ROW_NC, WIDTH_ODD>)
-                   : a.mult ? (even ? k_fire_warp<T, ROW_MULT, WIDTH_EVEN> : k_fire_warp<T, ROW_MULT, WIDTH_ODD>)
-                            : (even ? k_fire_warp<T, ROW_PLAIN, WIDTH_EVEN> : k_fire_warp<T, ROW_PLAIN, WIDTH_ODD>);
-    k<<<grid, 32 * kRowWarps, smem, s>>>(a);
+    row_kernel<T>(mode, even, full)<<<grid, 32 * kRowWarps, smem, s>>>(a);
     return cudaGetLastError();
 }
 
 #define WF_INSTANTIATE_WARP(T)                                          \
     template size_t warp_smem_bytes<T>(int, int, int);                  \
-    template cudaError_t prepare_warp_kernel<T>(size_t);                \
     template cudaError_t launch_warp<T>(const StepArgs &, cudaStream_t);
 
 }  // namespace wf
