@@ -1472,6 +1472,7 @@ int run_adjoint(fire_ctx *c, int nsteps, double dt, const void *u, const void *v
                 ctx_step_args(c, (pcur + s) & 1, u, v, dt, nullptr, nullptr, ra);
                 ra.psi_in = ck + (size_t)s * n;
                 ra.psi_out = ck + (size_t)(s + 1) * n;
+                ra.chained = s > 0;
                 e = launch_step_kernel(ra, cs);
             }
             StepArgs fin;
@@ -1712,6 +1713,7 @@ int run_adjoint(fire_ctx *c, int nsteps, double dt, const void *u, const void *v
             ra.t_in = tseg + j;
             ra.t_out = tseg + K + 1;
             ra.dt = dt;
+            ra.chained = j > 0;
             cudaError_t e = launch_step_kernel(ra, cs);
             if (e != cudaSuccess) return e;
         }

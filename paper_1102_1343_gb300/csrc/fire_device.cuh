@@ -13,6 +13,12 @@
 
 namespace wf {
 
+// in a kernel of launch_chained: its dependents may start; and, before it
+// touches what a step writes, the wait for the kernels before it (nothing
+// where it was launched the ordinary way)
+__device__ __forceinline__ void chain_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Index checks of the checked build (compiled with -DFIRE_BOUNDS_CHECK): an
 // index outside [0, n) sets ST_BOUNDS in the status variable st and becomes
 // 0, so the access stays inside its buffer and the kernel runs on (no trap,

@@ -81,7 +81,32 @@ struct StepArgs {
     // fuel fraction: 0 the subcell scheme of Sect. 3.3, 1 the scheme exact
     // for linear psi and t_i (2-D tile kernel only)
     int scheme;
+    // (host) the launch before on the stream is a kernel whose dependents may
+    // start early (launch_chained)
+    int chained;
 };
+
+// A launch that may start while the kernel before it on the stream still runs
+// (programmatic dependent launch): each of these kernels lets its dependents
+// start at once and waits for what it depends on itself before it touches
+// memory (chain_begin), so that one kernel's launch and the filling of the SMs
+// overlap the end of the one before.  Only for chains of the library's own
+// kernels (chained); after anything else the launch is an ordinary one.
+template <typename... P, typename... A>
+cudaError_t launch_chained(bool chained, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                           cudaStream_t s, const A &...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = chained ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
 
 struct IgnSeg {
     double ax, ay, bx, by;

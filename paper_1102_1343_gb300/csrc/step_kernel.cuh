@@ -146,11 +146,12 @@ __host__ __device__ inline size_t tile_wind_elems(int TX, int TY, int ky) {
 // more FP64 than the right-hand side); otherwise per node and stage.  Small
 // meshes, where this kernel is the default, are bound by the latency of its
 // chain of stages.  Measured, us per step (GB300), before and now: 100^2 nodes
-// in FP64 53.7 and 30.0.
+// in FP64 53.7 and 30.0 (25.7 with the tables formed during the step before).
 // ---------------------------------------------------------------------------
 template <typename T, bool TAB>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 : kTileCtasPerSmF32)
     k_fire_step(const StepArgs a) {
+    chain_go();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_status;
     const int tid = threadIdx.x;
@@ -178,10 +179,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 :
     T *wvx = wux + WR * BW2;
     T *rowt = wvx + WR * BW2;   // [4][BH2]: wind row and weight of u, of v
 
-    const T *__restrict__ psi_in = static_cast<const T *>(a.psi_in);
-    T *__restrict__ psi_out = static_cast<T *>(a.psi_out);
-    const T *__restrict__ F_in = static_cast<const T *>(a.F_in);
-    T *__restrict__ F_out = static_cast<T *>(a.F_out);
+    const T *psi_in = static_cast<const T *>(a.psi_in);
+    T *psi_out = static_cast<T *>(a.psi_out);
+    const T *F_in = static_cast<const T *>(a.F_in);
+    T *F_out = static_cast<T *>(a.F_out);
     const T *__restrict__ dzdx = static_cast<const T *>(a.dzdx);
     const T *__restrict__ dzdy = static_cast<const T *>(a.dzdy);
     const T *__restrict__ mult = static_cast<const T *>(a.mult);
@@ -214,24 +215,25 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 :
     const T idx = T(1) / T(a.dx), idy = T(1) / T(a.dy);
     const T i2dx = T(1) / (T(2) * T(a.dx)), i2dy = T(1) / (T(2) * T(a.dy));
     const T eps = T(a.eps);
-    const double tstart = *a.t_in;
-    const double t1 = tstart + a.dt;
     const int ncm1 = a.ncls - 1;
 
-    if (tid == 0) {
-        s_status = 0;
-        if (blockIdx.x == 0 && blockIdx.y == 0) *a.t_out = t1;
-    }
+    if (tid == 0) s_status = 0;
     int st = 0;
-    // ---- A: psi^n on the tile + 3 halo (0 outside the domain), the tables
-    for (int e = tid; e < BW3 * BH3; e += kThreads) {
-        int lx, ly;
-        split(e, BW3, lx, ly);
-        const int gy = y0 - 3 + ly, gx = x0 - 3 + lx;
-        T val = T(0);
-        if (gy >= 0 && gy < ny && gx >= 0 && gx < nx) val = psi_in[WF_CHK((size_t)gy * nx + gx, (long long)nx * ny, st)];
-        P0[e] = val;
-    }
+    // ---- A: psi^n on the tile + 3 halo (0 outside the domain), the tables, the
+    // node wind.  In a chained launch psi comes last: the rest does not wait
+    // for the step before.
+    auto load_psi = [&]() {
+        for (int e = tid; e < BW3 * BH3; e += kThreads) {
+            int lx, ly;
+            split(e, BW3, lx, ly);
+            const int gy = y0 - 3 + ly, gx = x0 - 3 + lx;
+            T val = T(0);
+            if (gy >= 0 && gy < ny && gx >= 0 && gx < nx)
+                val = psi_in[WF_CHK((size_t)gy * nx + gx, (long long)nx * ny, st)];
+            P0[e] = val;
+        }
+    };
+    if (!a.chained) load_psi();
     for (int k = tid; k < a.ncls * K_N; k += kThreads) lut[k] = T(a.coef[k]);
     const int jb = max(y0 / sry - 2, 0);  // first wind row of the table
     for (int e = tid; e < WR * BW2; e += kThreads) {
@@ -262,6 +264,29 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 :
         rowt[2 * BH2 + ly] = T(j0 - jb);
         rowt[3 * BH2 + ly] = wy;
     }
+    if constexpr (TAB) {
+        __syncthreads();
+        for (int e = tid; e < BW2 * BH2; e += kThreads) {
+            int lx, ly;
+            split(e, BW2, lx, ly);
+            // (rows past the last of u repeat it, with weight 0; frame nodes
+            // outside the mesh take the wind of its edge)
+            const T wyu = rowt[BH2 + ly], wyv = rowt[3 * BH2 + ly];
+            const T *u0 = wux + (int)rowt[ly] * BW2 + lx, *v0 = wvx + (int)rowt[2 * BH2 + ly] * BW2 + lx;
+            const T un = (T(1) - wyu) * u0[0] + wyu * u0[BW2];
+            const T vn = (T(1) - wyv) * v0[0] + wyv * v0[BW2];
+            if (!finite_val(un) || !finite_val(vn)) st |= ST_NONFINITE;
+            un_s[e] = un;
+            vn_s[e] = vn;
+        }
+    }
+    if (a.chained) {
+        chain_wait();
+        load_psi();
+    }
+    const double tstart = *a.t_in;
+    const double t1 = tstart + a.dt;
+    if (tid == 0 && blockIdx.x == 0 && blockIdx.y == 0) *a.t_out = t1;
     __syncthreads();
     const bool edge_tile = (x0 - 3 < 0) || (y0 - 3 < 0) || (x0 + TX + 3 > nx) || (y0 + TY + 3 > ny);
     if (edge_tile) fill_ghosts<T>(P0, BW3, BH3, x0 - 3, y0 - 3, nx, ny, tid);
@@ -278,19 +303,14 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 :
         const size_t g = WF_CHK((size_t)gy * nx + gx, (long long)nx * ny, st);
         int cls = fuel[g];
         cls = cls > ncm1 ? ncm1 : cls;
-        // the node's wind (rows past the last of u repeat it, with weight 0)
         T un, vn;
         if constexpr (TAB) {
-            const T wyu = rowt[BH2 + ly], wyv = rowt[3 * BH2 + ly];
-            const T *u0 = wux + (int)rowt[ly] * BW2 + lx, *v0 = wvx + (int)rowt[2 * BH2 + ly] * BW2 + lx;
-            un = (T(1) - wyu) * u0[0] + wyu * u0[BW2];
-            vn = (T(1) - wyv) * v0[0] + wyv * v0[BW2];
-            un_s[e] = un;
-            vn_s[e] = vn;
+            un = un_s[e];
+            vn = vn_s[e];
         } else {
             wind_at<T>(wu, wv, a.nxa, a.nya, srx, sry, gx, gy, un, vn, st);
+            if (!finite_val(un) || !finite_val(vn)) st |= ST_NONFINITE;
         }
-        if (!finite_val(un) || !finite_val(vn)) st |= ST_NONFINITE;
         const T m = mult ? mult[g] : T(1);
         const int c = (ly + 1) * BW3 + (lx + 1);
         T cn[6];
@@ -661,11 +681,8 @@ cudaError_t launch_step(const StepArgs &a, cudaStream_t s) {
     const size_t tab = step_table_bytes<T>(a.kx, a.ky, a.srx, a.sry, a.ncls);
     cudaError_t e = prepare_step_kernel<T>(smem);
     if (e != cudaSuccess) return e;
-    if (tab)
-        k_fire_step<T, true><<<grid, kThreads, tab, s>>>(a);
-    else
-        k_fire_step<T, false><<<grid, kThreads, smem, s>>>(a);
-    return cudaGetLastError();
+    return tab ? launch_chained(a.chained, k_fire_step<T, true>, grid, kThreads, tab, s, a)
+               : launch_chained(a.chained, k_fire_step<T, false>, grid, kThreads, smem, s, a);
 }
 
 template <typename T>
