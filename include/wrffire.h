@@ -466,9 +466,9 @@ int fire_step_noalloc(const fire_grid_desc *grid, const fire_fuel_class *classes
  * Batched ensemble: independent fire runs (different mesh sizes, fuels,
  * terrain, winds) advanced together.  Each fire_ensemble_step call runs all
  * members for nsteps steps in ONE persistent cooperative kernel launch (a
- * work list of member strips per step, a bounded grid-wide barrier between
- * steps), captured in a CUDA graph and replayed while its shape is
- * unchanged.  A member advanced here matches the same member advanced alone
+ * queue of member strips and steps, in which a strip waits, bounded, for its
+ * member's step before), captured in a CUDA graph and replayed while its shape
+ * is unchanged.  A member advanced here matches the same member advanced alone
  * by fire_step with the same kernel configuration.  Motivation: ensemble
  * data assimilation (Sect. 7, "Data assimilation"); not part of the paper's
  * fire step itself.
@@ -513,7 +513,7 @@ int fire_ensemble_step(fire_ensemble *ens, int nsteps, double dt, const void *co
  * fire_set_state, fire_status; do not destroy it). */
 int fire_ensemble_member(fire_ensemble *ens, int member, fire_ctx **ctx);
 
-/* Waits; returns FIRE_ERR_TIMEOUT if a barrier wait gave up, else the worst
+/* Waits; returns FIRE_ERR_TIMEOUT if a wait gave up, else the worst
  * member status; member_status (nullable host array [n]) receives each. */
 int fire_ensemble_status(fire_ensemble *ens, int *member_status);
 int fire_ensemble_clear_status(fire_ensemble *ens);
@@ -534,8 +534,8 @@ int fire_ensemble_autotune(fire_ensemble *ens, int probe_steps, double dt,
                            const void *const *wind_u_dev, const void *const *wind_v_dev,
                            int *strip_columns, int *strip_rows);
 
-/* Test hook for the bounded barrier: CTA skip_block (-1: none) never
- * arrives at the barriers, and waits give up after spin_limit polls (about
+/* Test hook for the bounded waits: CTA skip_block (-1: none) never
+ * reports its work done, and waits give up after spin_limit polls (about
  * 100 ns each), setting FIRE_ERR_TIMEOUT and ending the launch. */
 int fire_ensemble_set_barrier_test(fire_ensemble *ens, int skip_block, long long spin_limit);
 

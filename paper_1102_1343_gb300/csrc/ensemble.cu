@@ -1,21 +1,20 @@
 // Batched ensemble of independent fire runs (members of different mesh
 // sizes, fuels, winds) advanced together by ONE persistent cooperative
-// launch per call: the kernel loops over the steps, and within a step over
-// a work list of (member, strip) items handed out round-robin to the
-// resident CTAs; a grid-wide barrier separates the steps.  Each member is an
-// ordinary fire context (same state layout, same marching-strip device code
-// as fire_step), so a member advanced here matches the same member advanced
-// alone.  The launch (with the reset of the barrier word) is captured in a
+// launch per call: its resident CTAs take (member, strip, step) entries from a
+// queue, and an entry waits until its member has finished the step before
+// (EnsWork).  Each member is an ordinary fire context (same state layout, same
+// strip code as fire_step), so a member advanced here matches the same member
+// advanced alone.  The launch (with the reset of the queue) is captured in a
 // CUDA graph and replayed while its arguments do not change.
 //
-// Two forms of the persistent kernel, both with one (member, strip) item per
-// CTA at a time: FP32 ensembles run the strip code of k_fire_warp, FP64
-// ensembles (or refinements above 30) that of k_fire_march.
+// Two forms of the persistent kernel, both with one entry per CTA at a time:
+// FP32 ensembles run the strip code of k_fire_warp, FP64 ensembles (or
+// refinements above 30) that of k_fire_march.
 //
-// The barrier's wait is bounded: a CTA that waits longer than the spin limit
-// sets the ensemble's TIMEOUT bit and an abort flag, and every CTA leaves the
-// kernel at its next barrier, so a lost CTA ends the launch with an error
-// instead of hanging the device.
+// The waits are bounded: a CTA that waits longer than the spin limit sets the
+// status bit TIMEOUT and the abort flag, and every CTA leaves the kernel at its
+// next entry, so a lost CTA ends the launch with an error status instead of
+// hanging the GPU.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <string.h>
@@ -35,14 +34,16 @@ namespace {
 
 struct EnsItem {
     int member, x0, y0;
+    int count;  // items of the member
 };
 
-struct GridBar {
-    unsigned int count;
-    unsigned int gen;
+// the queue of a launch (zeroed before it, but for status): entry q is item
+// q mod n_items of step q / n_items
+struct EnsQueue {
+    int status;               // ensemble-wide status bits (TIMEOUT)
     int abort;
-    unsigned int next[2];  // work-item counters of alternate steps
-    int status;            // ensemble-wide status bits (TIMEOUT)
+    unsigned long long next;  // the first entry not handed out, less the grid
+    unsigned long long done[FIRE_MAX_MEMBERS];  // entries finished, per member
 };
 
 // values that change from call to call, read by the kernel from device memory
@@ -52,7 +53,7 @@ struct EnsRun {
     int parity0;
     int nsteps;
     long long spin_limit;
-    int skip_block;  // test hook: this CTA never arrives at a barrier (-1: none)
+    int skip_block;  // test hook: this CTA reports nothing done and ends (-1: none)
 };
 
 struct EnsembleArgs {
@@ -61,135 +62,131 @@ struct EnsembleArgs {
     int n_items;
     int n_members;
     double dt;
-    GridBar *bar;
+    EnsQueue *queue;
     const EnsRun *run;
 };
 
-// grid-wide barrier with a bounded wait; returns false when the launch must end
-__device__ bool grid_barrier(GridBar *b, long long spin_limit, bool skip) {
-    __shared__ int s_ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        volatile GridBar *vb = b;
-        bool ok = vb->abort == 0;
-        if (ok && !skip) {
-            const unsigned int g = vb->gen;
-            __threadfence();
-            const unsigned int arrived = atomicAdd(&b->count, 1u);
-            if (arrived == gridDim.x - 1) {
-                b->count = 0;
-                __threadfence();
-                atomicAdd(&b->gen, 1u);
-            } else {
-                long long it = 0;
-                while (vb->gen == g) {
-                    if (vb->abort) {
-                        ok = false;
-                        break;
-                    }
-                    if (++it > spin_limit) {
-                        atomicOr(&b->status, ST_TIMEOUT);
-                        atomicExch(&b->abort, 1);
-                        ok = false;
-                        break;
-                    }
-                    __nanosleep(100);
+// Work of the persistent kernels.  A step of a member needs the member's step
+// before, and nothing of the other members: entries are taken in order, and one
+// waits only until its member's entries of the step before are finished.  So
+// no step ends with an emptying device (a grid-wide barrier per step did: 24
+// members of 26..130 cells square, 40 steps, 13.7 ms; 13.0 so, and 11.7 with
+// the taller strips that this allows).  The lowest
+// unfinished entry never waits, so the queue always advances; the wait is
+// bounded all the same.  Entries are fetched one ahead.
+struct EnsWork {
+    unsigned long long q;  // current entry
+    unsigned long long ahead;  // thread 0: the next one
+    int step;
+    double t;
+
+    __device__ void start(const EnsRun &run) {
+        q = blockIdx.x;
+        step = 0;
+        t = run.t0;
+    }
+    // takes the current entry (all threads): false where the launch must end
+    __device__ bool take(const EnsembleArgs &e, const EnsRun &run, EnsItem &it) {
+        __shared__ int s_ok;
+        const unsigned long long total = (unsigned long long)e.n_items * run.nsteps;
+        if (q >= total) return false;
+        const int s = (int)(q / e.n_items);
+        it = e.items[q - (unsigned long long)s * e.n_items];
+        for (; step < s; ++step) t = t + e.dt;
+        if (threadIdx.x == 0) {
+            ahead = gridDim.x + atomicAdd(&e.queue->next, 1ull);
+            volatile EnsQueue *v = e.queue;
+            const unsigned long long need = (unsigned long long)s * it.count;
+            bool ok = v->abort == 0;
+            long long polls = 0;
+            while (ok && v->done[it.member] < need) {
+                if (v->abort) {
+                    ok = false;
+                    break;
                 }
+                if (++polls > run.spin_limit) {
+                    atomicOr(&e.queue->status, ST_TIMEOUT);
+                    atomicExch(&e.queue->abort, 1);
+                    ok = false;
+                    break;
+                }
+                __nanosleep(100);
             }
             __threadfence();
+            s_ok = ok;
         }
-        s_ok = ok;
+        __syncthreads();
+        return s_ok != 0;
     }
-    __syncthreads();
-    return s_ok != 0;
-}
+    // the entry is finished (all threads): false where the launch must end
+    __device__ bool finish(const EnsembleArgs &e, const EnsRun &run, const EnsItem &it) {
+        __shared__ unsigned long long s_next;
+        __syncthreads();
+        if ((int)blockIdx.x == run.skip_block) return false;
+        if (threadIdx.x == 0) {
+            __threadfence();
+            atomicAdd(&e.queue->done[it.member], 1ull);
+            s_next = ahead;
+        }
+        __syncthreads();
+        q = s_next;
+        return true;
+    }
+    // the members' device time after the last step
+    __device__ void end(const EnsembleArgs &e, const EnsRun &run) {
+        if (blockIdx.x != 0 || q < (unsigned long long)e.n_items * run.nsteps) return;
+        for (; step < run.nsteps; ++step) t = t + e.dt;
+        const int pf = (run.parity0 + run.nsteps) & 1;
+        for (int m = threadIdx.x; m < e.n_members; m += blockDim.x)
+            *const_cast<double *>(e.margs[2 * m + pf].t_in) = t;
+    }
+};
 
 template <typename T, bool NC>
 __global__ void __launch_bounds__(kMarchThreads, MarchOccupancy<T>::blocks)
     k_fire_ensemble(const EnsembleArgs e) {
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     const EnsRun run = *e.run;
-    double t = run.t0;
-    __shared__ int s_item;
-    for (int s = 0; s < run.nsteps; ++s) {
-        const int par = (run.parity0 + s) & 1;
-        // the counter of the next step was last used two steps ago
-        if (blockIdx.x == 0 && threadIdx.x == 0) e.bar->next[(s + 1) & 1] = 0;
-        for (;;) {
-            // items are taken dynamically, largest first (the list is sorted)
-            if (threadIdx.x == 0) s_item = (int)atomicAdd(&e.bar->next[s & 1], 1u);
-            __syncthreads();
-            const int i = s_item;
-            __syncthreads();
-            if (i >= e.n_items) break;
-            const EnsItem it = e.items[i];
-            const StepArgs &a = e.margs[2 * it.member + par];
-            MarchSmem<T> sm;
-            sm.carve(dyn_smem, a.ky * a.sry, a.ncls);
-            MarchStrip<T, NC> strip(a, sm);
-            strip.run(it.x0, it.y0, t);
-            if (strip.st) atomicOr(a.status, strip.st);
-            __syncthreads();  // shared memory is reused by the next item
-        }
-        t = t + e.dt;
-        if (s + 1 < run.nsteps) {
-            const bool skip = (int)blockIdx.x == run.skip_block;
-            if (!grid_barrier(e.bar, run.spin_limit, skip)) return;
-        }
+    EnsWork work;
+    EnsItem it;
+    for (work.start(run); work.take(e, run, it);) {
+        const StepArgs &a = e.margs[2 * it.member + ((run.parity0 + work.step) & 1)];
+        MarchSmem<T> sm;
+        sm.carve(dyn_smem, a.ky * a.sry, a.ncls);
+        MarchStrip<T, NC> strip(a, sm);
+        strip.run(it.x0, it.y0, work.t);
+        if (strip.st) atomicOr(a.status, strip.st);
+        if (!work.finish(e, run, it)) break;
     }
-    // the members' device time after the last step
-    if (blockIdx.x == 0) {
-        const int pf = (run.parity0 + run.nsteps) & 1;
-        for (int m = threadIdx.x; m < e.n_members; m += blockDim.x)
-            *const_cast<double *>(e.margs[2 * m + pf].t_in) = t;
-    }
+    work.end(e, run);
 }
 
 // the warp form: the CTA's warps share one item, its member's arguments in
 // shared memory.  One CTA per SM fewer than k_fire_warp: at 80 registers this
-// kernel spills 176 bytes (28 at 96): 24 members of 26..205 by 130 cells, 40
+// kernel spills 176 bytes (28 at 96): 24 members of 26..130 cells square, 40
 // steps, 14.35 ms with six CTAs, 13.69 with five (17.8 with the former kernel)
 template <typename T, int MODE, int WIDTH>
 __global__ void __launch_bounds__(32 * kRowWarps, (row_ctas<T, MODE>()) - 1)
     k_fire_ensemble_warp(const EnsembleArgs e) {
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     __shared__ StepArgs a;
-    __shared__ int s_item;
     RowSmem<T, kRowWarps> sm;
     const EnsRun run = *e.run;
-    double t = run.t0;
-    for (int s = 0; s < run.nsteps; ++s) {
-        const int par = (run.parity0 + s) & 1;
-        // the counter of the next step was last used two steps ago
-        if (blockIdx.x == 0 && threadIdx.x == 0) e.bar->next[(s + 1) & 1] = 0;
-        for (;;) {
-            // items are taken dynamically, largest first (the list is sorted)
-            if (threadIdx.x == 0) s_item = (int)atomicAdd(&e.bar->next[s & 1], 1u);
-            __syncthreads();
-            const int i = s_item;
-            if (i >= e.n_items) break;
-            const EnsItem it = e.items[i];
-            const int *src = reinterpret_cast<const int *>(e.margs + 2 * it.member + par);
-            for (int q = threadIdx.x; q < (int)(sizeof(StepArgs) / sizeof(int)); q += 32 * kRowWarps)
-                reinterpret_cast<int *>(&a)[q] = src[q];
-            __syncthreads();
-            sm.carve(dyn_smem, a.ky, a.sry, a.ncls);
-            RowStrip<T, MODE, kRowWarps, WIDTH> strip(a, sm, dyn_smem);
-            strip.run(it.x0, it.y0, t);  // ends with a barrier
-            const int stw = __reduce_or_sync(0xffffffffu, strip.st);
-            if ((threadIdx.x & 31) == 0 && stw) atomicOr(a.status, stw);
-        }
-        t = t + e.dt;
-        if (s + 1 < run.nsteps) {
-            const bool skip = (int)blockIdx.x == run.skip_block;
-            if (!grid_barrier(e.bar, run.spin_limit, skip)) return;
-        }
+    EnsWork work;
+    EnsItem it;
+    for (work.start(run); work.take(e, run, it);) {
+        const int *src = reinterpret_cast<const int *>(e.margs + 2 * it.member + ((run.parity0 + work.step) & 1));
+        for (int q = threadIdx.x; q < (int)(sizeof(StepArgs) / sizeof(int)); q += 32 * kRowWarps)
+            reinterpret_cast<int *>(&a)[q] = src[q];
+        __syncthreads();
+        sm.carve(dyn_smem, a.ky, a.sry, a.ncls);
+        RowStrip<T, MODE, kRowWarps, WIDTH> strip(a, sm, dyn_smem);
+        strip.run(it.x0, it.y0, work.t);  // ends with a barrier
+        const int stw = __reduce_or_sync(0xffffffffu, strip.st);
+        if ((threadIdx.x & 31) == 0 && stw) atomicOr(a.status, stw);
+        if (!work.finish(e, run, it)) break;
     }
-    if (blockIdx.x == 0) {
-        const int pf = (run.parity0 + run.nsteps) & 1;
-        for (int m = threadIdx.x; m < e.n_members; m += blockDim.x)
-            *const_cast<double *>(e.margs[2 * m + pf].t_in) = t;
-    }
+    work.end(e, run);
 }
 
 }  // namespace
@@ -224,7 +221,7 @@ struct fire_ensemble {
     StepArgs *margs_host = nullptr;  // pinned
     EnsItem *items_dev = nullptr;
     int n_items = 0;
-    GridBar *bar = nullptr;
+    EnsQueue *queue = nullptr;
     EnsRun *run_dev = nullptr;
     EnsRun *run_host = nullptr;  // pinned
     cudaEvent_t staged = nullptr;  // the pinned staging buffers may be rewritten
@@ -270,7 +267,7 @@ void ens_release(fire_ensemble *e) {
     for (fire_ctx *c : e->members) fire_destroy(c);
     if (e->margs_dev) cudaFree(e->margs_dev);
     if (e->items_dev) cudaFree(e->items_dev);
-    if (e->bar) cudaFree(e->bar);
+    if (e->queue) cudaFree(e->queue);
     if (e->run_dev) cudaFree(e->run_dev);
     if (e->margs_host) cudaFreeHost(e->margs_host);
     if (e->run_host) cudaFreeHost(e->run_host);
@@ -296,7 +293,8 @@ int ens_plan(fire_ensemble *e) {
         cudaGraphExecDestroy(e->graph);
         e->graph = nullptr;
     }
-    std::vector<EnsItem> items;
+    // a member's items one after the other, the largest member first
+    std::vector<std::vector<EnsItem>> of(e->n);
     size_t smem = 0;
     for (int m = 0; m < e->n; ++m) {
         int prec, variant, nx, ny, srx, sry, kx, ky, ncls, cur;
@@ -305,8 +303,9 @@ int ens_plan(fire_ensemble *e) {
         if (variant != e->variant) return FIRE_ERR_STATE;
         if (e->variant == FIRE_KERNEL_WARP) ky = row_strip_bands(ky, sry);
         const int W = kx * srx, L = ky * sry;
+        const int count = ((nx + W - 1) / W) * ((ny + L - 1) / L);
         for (int y0 = 0; y0 < ny; y0 += L)
-            for (int x0 = 0; x0 < nx; x0 += W) items.push_back(EnsItem{m, x0, y0});
+            for (int x0 = 0; x0 < nx; x0 += W) of[m].push_back(EnsItem{m, x0, y0, count});
         if (e->variant == FIRE_KERNEL_MARCH) {
             const size_t sm = e->prec == FIRE_FP64 ? march_smem_bytes<double>(ky, sry, ncls)
                                                    : march_smem_bytes<float>(ky, sry, ncls);
@@ -317,29 +316,11 @@ int ens_plan(fire_ensemble *e) {
             smem = std::max(smem, sm);
         }
     }
-    // largest items first (the kernel hands them out dynamically), then by
-    // row and member
-    std::vector<long long> cost(items.size());
-    for (size_t q = 0; q < items.size(); ++q) {
-        int prec, variant, nx, ny, srx, sry, kx, ky, ncls, cur;
-        double t;
-        ctx_info(e->members[items[q].member], &prec, &variant, &nx, &ny, &srx, &sry, &kx, &ky,
-                 &ncls, &cur, &t);
-        if (e->variant == FIRE_KERNEL_WARP) ky = row_strip_bands(ky, sry);
-        cost[q] = (long long)std::min(kx * srx, nx - items[q].x0) * std::min(ky * sry, ny - items[q].y0);
-    }
-    std::vector<size_t> order(items.size());
-    for (size_t q = 0; q < order.size(); ++q) order[q] = q;
-    std::stable_sort(order.begin(), order.end(), [&](size_t a, size_t b) {
-        if (cost[a] != cost[b]) return cost[a] > cost[b];
-        if (items[a].y0 != items[b].y0) return items[a].y0 < items[b].y0;
-        return items[a].member < items[b].member;
+    std::stable_sort(of.begin(), of.end(), [](const std::vector<EnsItem> &a, const std::vector<EnsItem> &b) {
+        return a.size() > b.size();
     });
-    {
-        std::vector<EnsItem> sorted(items.size());
-        for (size_t q = 0; q < order.size(); ++q) sorted[q] = items[order[q]];
-        items.swap(sorted);
-    }
+    std::vector<EnsItem> items;
+    for (const std::vector<EnsItem> &o : of) items.insert(items.end(), o.begin(), o.end());
     if (e->items_dev) cudaFree(e->items_dev);
     e->items_dev = nullptr;
     ENS_CHECK(cudaMalloc(&e->items_dev, sizeof(EnsItem) * items.size()));
@@ -390,9 +371,9 @@ cudaError_t ens_launch(fire_ensemble *e, double dt, cudaStream_t s) {
     ea.n_items = e->n_items;
     ea.n_members = e->n;
     ea.dt = dt;
-    ea.bar = e->bar;
+    ea.queue = e->queue;
     ea.run = e->run_dev;
-    cudaError_t err = cudaMemsetAsync(e->bar, 0, offsetof(GridBar, status), s);
+    cudaError_t err = cudaMemsetAsync(&e->queue->abort, 0, sizeof(EnsQueue) - offsetof(EnsQueue, abort), s);
     if (err != cudaSuccess) return err;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof cfg);
@@ -457,8 +438,13 @@ int fire_ensemble_create(fire_ensemble **out, int n_members, const fire_member_d
     // the warp form when every member can take warp strips (FP32, refinement
     // <= 30), else the marching form for all; members start from marching
     // strips of the large-mesh size, or from warp strips whose height suits
-    // the whole ensemble: the items of a step are handed out to the CTAs as
-    // warp_launch_rows' CTAs are to the SMs, so the same cost is least
+    // the whole ensemble.  A step costs its items times L + 23 rows' time over
+    // the resident CTAs, and, where the largest member's next step follows
+    // within a wave or two, waits of up to 0.8 (L + 20).  Measured, ms per 40
+    // steps: 24 members of 26..130 cells square, rows 60: 13.0, 80: 12.4, 120:
+    // 11.7 (taken), 160: 11.4; 60 members of 26..40, rows 40: 8.3, 60: 7.6
+    // (taken), 80: 7.2, 120: 7.4; 3 members of 100..130, rows 30: 3.4, 40: 3.1
+    // (taken), 60: 3.1, 80: 3.5.
     if (r == FIRE_OK) {
         bool warp = prec == FIRE_FP32;
         for (fire_ctx *c : e->members) {
@@ -472,14 +458,20 @@ int fire_ensemble_create(fire_ensemble **out, int n_members, const fire_member_d
         int rows = 10, n_sm = 1;
         double least = 0;
         r = ens_cuda(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, e->device));
+        const double slots = (double)n_sm * (kRowCtasPerSmF32 - 1);
         for (int L = 10; L <= 160; L += 10) {
-            double t = 0;
+            double all = 0, most = 0;
             for (fire_ctx *c : e->members) {
                 int nx = 0, ny = 0;
                 fire_mesh_size(c, &nx, &ny);
-                t += (double)((nx + kWarpMaxColumns - 1) / kWarpMaxColumns) * ((ny + L - 1) / L);
+                const double own =
+                    (double)((nx + kWarpMaxColumns - 1) / kWarpMaxColumns) * ((ny + L - 1) / L);
+                all += own;
+                most = std::max(most, own);
             }
-            t = t * (L + 10) / ((double)n_sm * kRowCtasPerSmF32) + 0.8 * (L + 20);
+            const double between = (all - most) / slots;  // waves from a member's step to its next
+            const double wait = std::min(0.8, std::max(0.0, 0.8 - 0.4 * (between - 1.0)));
+            const double t = all * (L + 23) / slots + wait * (L + 20);
             if (L == 10 || t < least) {
                 least = t;
                 rows = L;
@@ -495,11 +487,11 @@ int fire_ensemble_create(fire_ensemble **out, int n_members, const fire_member_d
     } while (0)
     ENS_TRY(cudaMalloc(&e->margs_dev, sizeof(StepArgs) * 2 * n_members));
     ENS_TRY(cudaMallocHost(&e->margs_host, sizeof(StepArgs) * 2 * n_members));
-    ENS_TRY(cudaMalloc(&e->bar, sizeof(GridBar)));
+    ENS_TRY(cudaMalloc(&e->queue, sizeof(EnsQueue)));
     ENS_TRY(cudaMalloc(&e->run_dev, sizeof(EnsRun)));
     ENS_TRY(cudaMallocHost(&e->run_host, sizeof(EnsRun)));
     ENS_TRY(cudaEventCreateWithFlags(&e->staged, cudaEventDisableTiming));
-    ENS_TRY(cudaMemsetAsync(e->bar, 0, sizeof(GridBar), e->stream));
+    ENS_TRY(cudaMemsetAsync(e->queue, 0, sizeof(EnsQueue), e->stream));
 #undef ENS_TRY
     if (r == FIRE_OK) r = ens_plan(e);
     if (r == FIRE_OK) r = ens_cuda(cudaStreamSynchronize(e->stream));
@@ -627,8 +619,8 @@ int fire_ensemble_status(fire_ensemble *e, int *member_status) {
     if (!e) return FIRE_ERR_ARG;
     DeviceGuard dg(e->device);
     ENS_CHECK(cudaStreamSynchronize(e->stream));
-    GridBar b;
-    ENS_CHECK(cudaMemcpy(&b, e->bar, sizeof b, cudaMemcpyDeviceToHost));
+    int ens_status = 0;
+    ENS_CHECK(cudaMemcpy(&ens_status, &e->queue->status, sizeof ens_status, cudaMemcpyDeviceToHost));
     int worst = FIRE_OK;
     for (int m = 0; m < e->n; ++m) {
         const int s = fire_status(e->members[m]);
@@ -637,7 +629,7 @@ int fire_ensemble_status(fire_ensemble *e, int *member_status) {
             (worst == FIRE_OK || s == FIRE_ERR_NONFINITE || s == FIRE_ERR_BOUNDS))
             worst = s;
     }
-    if (b.status & ST_TIMEOUT) return FIRE_ERR_TIMEOUT;
+    if (ens_status & ST_TIMEOUT) return FIRE_ERR_TIMEOUT;
     return worst;
 }
 
@@ -647,7 +639,7 @@ int fire_ensemble_clear_status(fire_ensemble *e) {
         int r = fire_clear_status(c);
         if (r) return r;
     }
-    ENS_CHECK(cudaMemsetAsync(e->bar, 0, sizeof(GridBar), e->stream));
+    ENS_CHECK(cudaMemsetAsync(e->queue, 0, sizeof(EnsQueue), e->stream));
     return FIRE_OK;
 }
 
