@@ -294,7 +294,13 @@ int apply_ignitions(fire_ctx *c, const std::vector<IgnSeg> &segs) {
         a.dx = c->dx;
         a.dy = c->dy;
         int m = 0;
-        while (k < segs.size() && m < kMaxSegPerLaunch) a.seg[m++] = segs[k++];
+        while (k < segs.size() && m < kMaxSegPerLaunch) {
+            IgnSeg &q = a.seg[m++] = segs[k++];
+            q.dx = q.bx - q.ax;
+            q.dy = q.by - q.ay;
+            const double l2 = q.dx * q.dx + q.dy * q.dy;
+            q.il2 = l2 > 0.0 ? 1.0 / l2 : 0.0;
+        }
         a.nseg = m;
         cudaError_t e = c->prec == FIRE_FP64 ? launch_ignite<double>(a, c->stream)
                                              : launch_ignite<float>(a, c->stream);

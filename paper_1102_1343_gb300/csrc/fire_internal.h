@@ -116,6 +116,8 @@ struct IgnSeg {
     // parameter u of [a, b] was laid at tg + u (tlay - tg)
     int drip;
     double tnow, tlay;
+    // b - a, and 1/|b - a|^2 (0 for a point); set by apply_ignitions
+    double dx, dy, il2;
 };
 
 struct IgniteArgs {

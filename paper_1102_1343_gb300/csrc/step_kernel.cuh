@@ -472,11 +472,12 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 :
 // cover a node (then it may set the ignition time, which does): the others
 // are left out for the whole tile, and a tile with none left is done without
 // a look at its ignition times.  The exact test in double runs only where one
-// in float, with its rounding bounded, cannot exclude it.  Bound by reading psi
-// where no segment is near.  On a 1400x1000 mesh with four drip torches the
-// kernel took 163 us before, every node testing every segment with differences
-// in double on the narrow FP64 pipe; a step with it now takes 111 us instead
-// of 210.
+// in float, with its rounding bounded, cannot exclude it: near a moving torch
+// that is every node it is the nearest fire of, and their FP64 operations (some
+// 18, with the quotient by |b - a|^2 a product, the limits on the bits and the
+// root of sqrt64) bound the kernel; elsewhere reading psi does.  On a 1400x1000 mesh with four drip torches the
+// kernel took 163 us when every node tested every segment in double, 59 with
+// the exact test's IEEE quotient and root; a step with it takes 69 us (210, 94).
 // ---------------------------------------------------------------------------
 constexpr int kIgnX = 64, kIgnY = 16, kIgnThreads = 256, kIgnPer = kIgnX * kIgnY / kIgnThreads;
 static_assert(kMaxSegPerLaunch <= kIgnThreads, "one thread bounds each segment of a launch");
@@ -516,7 +517,7 @@ __global__ void __launch_bounds__(kIgnThreads) k_ignite(const IgniteArgs a) {
     if (tid < a.nseg) {
         const IgnSeg &s = a.seg[tid];
         const float qx = (float)(xc - s.ax), qy = (float)(yc - s.ay);
-        const float sx = (float)(s.bx - s.ax), sy = (float)(s.by - s.ay);
+        const float sx = (float)s.dx, sy = (float)s.dy;
         const float L2 = sx * sx + sy * sy;
         float u = L2 > 0.0f ? (qx * sx + qy * sy) / L2 : 0.0f;
         u = fminf(fmaxf(u, 0.0f), 1.0f);
@@ -560,6 +561,7 @@ __global__ void __launch_bounds__(kIgnThreads) k_ignite(const IgniteArgs a) {
     __syncthreads();
     const int n = s_n;
     if (n == 0 || i >= a.nx) return;
+    const double x = ((double)i + 0.5) * a.dx;
 #pragma unroll
     for (int e = 0; e < kIgnPer; ++e) {
         const int jl = ly + e * (kIgnThreads / kIgnX), j = y0 + jl;
@@ -567,6 +569,7 @@ __global__ void __launch_bounds__(kIgnThreads) k_ignite(const IgniteArgs a) {
         const float ox = ((float)lx + 0.5f - 0.5f * kIgnX) * (float)a.dx, oy = ((float)jl + 0.5f - 0.5f * kIgnY) * (float)a.dy;
         const size_t g = (size_t)j * a.nx + i;
         T pe = p[e];
+        const double y = ((double)j + 0.5) * a.dy;
         double ti = 0.0;
         bool read = false, changed = false, tchanged = false;
         for (int q = 0; q < n; ++q) {
@@ -578,7 +581,7 @@ __global__ void __launch_bounds__(kIgnThreads) k_ignite(const IgniteArgs a) {
             // distance in float
             {
                 const float qx = s_qx[k] + ox, qy = s_qy[k] + oy;
-                const float sx = (float)(s.bx - s.ax), sy = (float)(s.by - s.ay);
+                const float sx = (float)s.dx, sy = (float)s.dy;
                 const float L2f = sx * sx + sy * sy;
                 float u = L2f > 0.0f ? (qx * sx + qy * sy) / L2f : 0.0f;
                 u = fminf(fmaxf(u, 0.0f), 1.0f);
@@ -589,19 +592,15 @@ __global__ void __launch_bounds__(kIgnThreads) k_ignite(const IgniteArgs a) {
                 const float dl = lim + delta + 1e-6f * fabsf(lim);
                 if (!(dl > 0.0f && !(d2 > dl * dl))) continue;
             }
-            const double x = ((double)i + 0.5) * a.dx, y = ((double)j + 0.5) * a.dy;
-            const double dxs = s.bx - s.ax, dys = s.by - s.ay;
             const double qx = x - s.ax, qy = y - s.ay;
-            const double L2 = dxs * dxs + dys * dys;
-            double u = 0.0;
-            if (L2 > 0.0) {
-                u = (qx * dxs + qy * dys) / L2;
-                u = u < 0.0 ? 0.0 : (u > 1.0 ? 1.0 : u);
-            }
-            const double rx = qx - u * dxs, ry = qy - u * dys;
-            const double d = sqrt(rx * rx + ry * ry);
+            double u = (qx * s.dx + qy * s.dy) * s.il2;
+            // u limited to [0, 1] on its bits
+            if (__double_as_longlong(u) <= 0) u = 0.0;
+            else if (__double2hiint(u) >= 0x3ff00000) u = 1.0;
+            const double rx = qx - u * s.dx, ry = qy - u * s.dy;
+            const double d = sqrt64(rx * rx + ry * ry);
             const double pg = d - s.rho;
-            if ((double)pe > 0.0 && pg <= 0.0) {
+            if (pe > T(0) && le0(pg)) {
                 if (!read) {
                     ti = a.tign[g];
                     read = true;
@@ -618,8 +617,10 @@ __global__ void __launch_bounds__(kIgnThreads) k_ignite(const IgniteArgs a) {
                     tchanged = true;
                 }
             }
-            if (pg < (double)pe) {
-                pe = T(pg);
+            // (pg < psi where the rounded pg is: an equal one changes nothing)
+            const T pt = T(pg);
+            if (pt < pe) {
+                pe = pt;
                 changed = true;
             }
         }
