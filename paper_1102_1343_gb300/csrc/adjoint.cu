@@ -1118,12 +1118,16 @@ __device__ void quad_partials(const double *w, const double *th, double t1, doub
     // midpoints and the four corners, indexed by window position 3b + a
     double vp[9], vt[9];
     int vn[9][4], vc[9];
+#pragma unroll
     for (int b = 0; b < 3; ++b)
+#pragma unroll
         for (int a = 0; a < 3; ++a) {
             const int v = 3 * b + a, xs[2] = {a == 0 ? 0 : 1, a == 2 ? 2 : 1},
                       ys[2] = {b == 0 ? 0 : 1, b == 2 ? 2 : 1};
             int m = 0;
+#pragma unroll
             for (int yy = 0; yy < (ys[0] == ys[1] ? 1 : 2); ++yy)
+#pragma unroll
                 for (int xx = 0; xx < (xs[0] == xs[1] ? 1 : 2); ++xx) vn[v][m++] = 3 * ys[yy] + xs[xx];
             vc[v] = m;
             double sp = 0.0, st = 0.0;
@@ -1141,10 +1145,12 @@ __device__ void quad_partials(const double *w, const double *th, double t1, doub
             vt[v] = sp >= 0.0 ? t1 : st;
         }
     double gv[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, gt[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+#pragma unroll
     for (int sub = 0; sub < 4; ++sub) {
         const int cx = (sub & 1) ? 2 : 0, cy = (sub & 2) ? 2 : 0;
         const int vs[4] = {4, 3 + cx, 3 * cy + 1, 3 * cy + cx};  // centre, x-edge, y-edge, corner
         double s = 0.0, a = 0.0, tau = 0.0;
+#pragma unroll
         for (int q = 0; q < 4; ++q) {
             s += vp[vs[q]];
             a += fabs(vp[vs[q]]);
@@ -1152,6 +1158,7 @@ __device__ void quad_partials(const double *w, const double *th, double t1, doub
         }
         const double e = exp(-0.25 * tau / Tf);
         const double beta = a > 0.0 ? 0.5 * (1.0 - s / a) : 0.0;
+#pragma unroll
         for (int q = 0; q < 4; ++q) {
             const double x = vp[vs[q]];
             const double sg = x > 0.0 ? 1.0 : (x < 0.0 ? -1.0 : 0.0);
@@ -1161,12 +1168,15 @@ __device__ void quad_partials(const double *w, const double *th, double t1, doub
             gt[vs[q]] += 0.0625 * beta * e / Tf;
         }
     }
+#pragma unroll
     for (int q = 0; q < 9; ++q) {
         dw[q] = 0.0;
         dth[q] = 0.0;
     }
+#pragma unroll
     for (int v = 0; v < 9; ++v) {
         const double f = 1.0 / vc[v];
+#pragma unroll
         for (int m = 0; m < vc[v]; ++m) {
             dw[vn[v][m]] += f * gv[v];
             if (vp[v] < 0.0) dth[vn[v][m]] += f * gt[v];
@@ -1183,7 +1193,10 @@ __device__ bool heat_cell(const HeatArgs<T> &h, int i, int j, double *dw, double
     const double g = h.gF[k];
     if (g == 0.0) return false;
     double th[9];
+    bool any = false;
+#pragma unroll
     for (int b = 0; b < 3; ++b)
+#pragma unroll
         for (int a = 0; a < 3; ++a) {
             const int x = i + a - 1, y = j + b - 1;
             const double p = ext_psi(h.psi, h.nx, h.ny, x, y);
@@ -1193,7 +1206,10 @@ __device__ bool heat_cell(const HeatArgs<T> &h, int i, int j, double *dw, double
             const size_t kc = (size_t)yc * h.nx + xc;
             w[3 * b + a] = p;
             th[3 * b + a] = (p >= 0.0 || !((double)h.psi[kc] < 0.0)) ? h.t1 : h.tign[kc];
+            any |= !(p >= 0.0);
         }
+    // no psi < 0 in the window: beta = 0 and 1 - e = 0, all contributions are 0
+    if (!any) return false;
     const size_t c = (size_t)min((int)h.fuel[k], h.ncls - 1);
     quad_partials(w, th, h.t1, h.coef[c * K_N + K_TF], dw, dth);
     for (int q = 0; q < 9; ++q) {
@@ -1205,41 +1221,49 @@ __device__ bool heat_cell(const HeatArgs<T> &h, int i, int j, double *dw, double
 
 // per node: the contributions of the (up to 9) cells whose window holds the
 // node itself (the ghost positions of the boundary cells are added by
-// k_heat_ghosts).  A cell whose window has no psi < 0 contributes exact zeros
-// (beta = 0 and 1 - e = 0), so inside the mesh a node whose 5x5
-// neighbourhood has none is done: on a 370x290 mesh with a fire of 60 m this
-// took the kernel, bound by the nine FP64 quadratures per node, from 2612 us
-// to a few tens
+// k_heat_ghosts).  A CTA forms the quadratures of a tile's cells and of those
+// around it once, a cell per thread, in shared memory, and its nodes add theirs
+// in a fixed order; a tile whose cells' windows have no psi < 0 has none.  With
+// nine quadratures one after the other in every node's thread the kernel,
+// bound by the latency of that chain, took 978 us on a 370x290 mesh with a fire
+// of 60 m; 60 steps there and their adjoint take 2.27 ms instead of 3.54 with
+// this form and what k_heat_ghosts leaves out.
+constexpr int kHgX = 16, kHgY = 8, kHgCells = (kHgX + 2) * (kHgY + 2), kHgThreads = 192;
+
 template <typename T>
-__global__ void k_heat_gather(const HeatArgs<T> h) {
-    const size_t n = (size_t)h.nx * h.ny;
-    for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < n;
-         k += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(k % h.nx), j = (int)(k / h.nx);
-        if (i >= 2 && i < h.nx - 2 && j >= 2 && j < h.ny - 2) {
-            bool any = false;
-            for (int dy = -2; dy <= 2; ++dy)
-                for (int dx = -2; dx <= 2; ++dx) any |= !(h.psi[k + (ptrdiff_t)dy * h.nx + dx] >= T(0));
-            if (!any) {
-                h.lamd[k] = 0.0;
-                h.dJdt[k] = 0.0;
-                continue;
-            }
+__global__ void __launch_bounds__(kHgThreads) k_heat_gather(const HeatArgs<T> h) {
+    __shared__ double s_w[9][kHgCells], s_t[9][kHgCells];
+    const int tx = (h.nx + kHgX - 1) / kHgX, tid = threadIdx.x;
+    const int x0 = (int)(blockIdx.x % tx) * kHgX, y0 = (int)(blockIdx.x / tx) * kHgY;
+    bool on = false;
+    if (tid < kHgCells) {
+        const int ci = x0 - 1 + tid % (kHgX + 2), cj = y0 - 1 + tid / (kHgX + 2);
+        double dw[9], dth[9], w[9];
+        on = ci >= 0 && ci < h.nx && cj >= 0 && cj < h.ny && heat_cell(h, ci, cj, dw, dth, w);
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            s_w[q][tid] = on ? dw[q] : 0.0;
+            s_t[q][tid] = on ? dth[q] : 0.0;
         }
+    }
+    on = __syncthreads_or(on);
+    const int i = x0 + tid % kHgX, j = y0 + tid / kHgX;
+    if (tid >= kHgX * kHgY || i >= h.nx || j >= h.ny) return;
+    const size_t k = (size_t)j * h.nx + i;
+    double lp = 0.0, lt = 0.0;
+    if (on) {
         const bool tnode = (double)h.psi[k] < 0.0;
-        double lp = 0.0, lt = 0.0, dw[9], dth[9], w[9];
         for (int dy = -1; dy <= 1; ++dy)
             for (int dx = -1; dx <= 1; ++dx) {
-                const int ci = i - dx, cj = j - dy;  // cell whose window has this node at (dx, dy)
-                if (ci < 0 || ci >= h.nx || cj < 0 || cj >= h.ny) continue;
-                if (!heat_cell(h, ci, cj, dw, dth, w)) continue;
+                // the cell whose window has this node at (dx, dy)
+                const int c = (tid / kHgX + 1 - dy) * (kHgX + 2) + tid % kHgX + 1 - dx;
                 const int q = 3 * (dy + 1) + (dx + 1);
-                lp += dw[q];
-                if (tnode) lt += dth[q];
+                lp += s_w[q][c];
+                if (tnode) lt += s_t[q][c];
             }
-        h.lamd[k] = lp;
-        h.dJdt[k] = lt;
     }
+    h.lamd[k] = lp;
+    h.dJdt[k] = lt;
 }
 
 // d(psi at position (x, y) of the ghost-extended mesh)/d(psi of node (i, j)):
@@ -1270,7 +1294,8 @@ __device__ double ext_partial(const T *psi, int nx, int ny, int x, int y, int i,
 // extrapolate; t^ ghosts: the node they copy), cells in a fixed order.  The
 // cells concerned are boundary cells within one node.  (One thread for the
 // whole boundary took 50 ms on a 370x290 mesh, the chain of 1316 FP64
-// quadratures one after the other.)
+// quadratures one after the other; 405 us with all cells' quadratures, those
+// of unburnt windows too.)
 template <typename T>
 __global__ void k_heat_ghosts(const HeatArgs<T> h) {
     const int nx = h.nx, ny = h.ny;
@@ -1693,7 +1718,8 @@ int run_adjoint(fire_ctx *c, int nsteps, double dt, const void *u, const void *v
         h.lamd = hs + n;
         h.dJdt = hs + 2 * n;
         k_heat_seed<T><<<grid, kAdjThreads, 0, st>>>(h);
-        k_heat_gather<T><<<grid, kAdjThreads, 0, st>>>(h);
+        const size_t hg = ((size_t)(nx + kHgX - 1) / kHgX) * ((size_t)(ny + kHgY - 1) / kHgY);
+        k_heat_gather<T><<<(unsigned)hg, kHgThreads, 0, st>>>(h);
         const long ring = 4L * ((long)nx + ny);  // at least the nodes of the two outer rings
         k_heat_ghosts<T><<<(int)((ring + 63) / 64), 64, 0, st>>>(h);
         k_heat_lambda<T><<<grid, kAdjThreads, 0, st>>>(h.lamd, lam, n);
