@@ -167,6 +167,9 @@ __device__ __forceinline__ bool any_sign(float a, float b, float c) {
 }
 __device__ __forceinline__ bool nonzero(float x) { return x != 0.0f; }
 __device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
+// a number below 0 among three (FP64: a set sign)
+__device__ __forceinline__ bool any_neg(float a, float b, float c) { return fminf(fminf(a, b), c) < 0.0f; }
+__device__ __forceinline__ bool any_neg(double a, double b, double c) { return any_sign(a, b, c); }
 // x <= 0
 __device__ __forceinline__ bool le0(float x) { return x <= 0.0f; }
 __device__ __forceinline__ bool le0(double x) { return __double_as_longlong(x) <= 0; }
@@ -335,6 +338,38 @@ __device__ __forceinline__ T cell_fraction_vals(T p00, T p01, T p02, T p10, T p1
     T bNE = subcell_burned<T>(p11, pE, pN, pNE, dC, dE, dN, dNE, k);
     // one fused multiply-add, as in the packed two-cell version
     return fma(-q, ((bSW + bSE) + bNW) + bNE, T(1));
+}
+
+// The burned fractions of the two subcells below (side 0) or above (side 1) the
+// cell's centre row, west then east, with the operations of
+// cell_fraction_vals: node c of P and D (rows S apart), zeros where the
+// neighbourhood has no burning node.
+template <typename T>
+__device__ __forceinline__ void cell_fraction_half(const T *P, const T *D, int c, int S, int side, T Tf,
+                                                   T &bW, T &bE) {
+    bW = bE = T(0);
+    const int o = side ? c + S : c - S, x = side ? c - S : c + S;  // this side's row, the other
+    const T o0 = P[o - 1], o1 = P[o], o2 = P[o + 1], m0 = P[c - 1], m1 = P[c], m2 = P[c + 1];
+    if (!any_neg(o0, o1, o2) && !any_neg(m0, m1, m2) && !any_neg(P[x - 1], P[x], P[x + 1])) return;
+    const T e0 = D[o - 1], e1 = D[o], e2 = D[o + 1], f0 = D[c - 1], f1 = D[c], f2 = D[c + 1];
+    const T h = T(0.5), q = T(0.25);
+    T pW = h * (m0 + m1), pE = h * (m1 + m2), pO = h * (o1 + m1);
+    T dW = h * (f0 + f1), dE = h * (f1 + f2), dO = h * (e1 + f1);
+    // corners: the lower row's two nodes first
+    auto corner = [&](T oa, T ob, T ma, T mb) {
+        return q * (side ? ((ma + mb) + oa) + ob : ((oa + ob) + ma) + mb);
+    };
+    T pCW = corner(o0, o1, m0, m1), pCE = corner(o1, o2, m1, m2);
+    T dCW = corner(e0, e1, f0, f1), dCE = corner(e1, e2, f1, f2);
+    const T dC = m1 >= T(0) ? T(0) : f1;
+    dW = pW >= T(0) ? T(0) : dW;
+    dE = pE >= T(0) ? T(0) : dE;
+    dO = pO >= T(0) ? T(0) : dO;
+    dCW = pCW >= T(0) ? T(0) : dCW;
+    dCE = pCE >= T(0) ? T(0) : dCE;
+    const T k = T(-0.25) / Tf;
+    bW = subcell_burned<T>(m1, pW, pO, pCW, dC, dW, dO, dCW, k);
+    bE = subcell_burned<T>(m1, pE, pO, pCE, dC, dE, dO, dCE, k);
 }
 
 // ---------------------------------------------------------------------------

@@ -99,16 +99,6 @@ __device__ void fill_ghosts_pd(T *P, T *Dl, int BW, int BH, int ox, int oy, int 
     __syncthreads();
 }
 
-// Fuel fraction of the cell at index c of the staged psi^{n+1} (P) and
-// Dl = t - t_i (row pitch W).
-template <typename T>
-__device__ __forceinline__ T cell_fraction(const T *P, const T *Dl, int c, int W, T Tf) {
-    return cell_fraction_vals<T>(P[c - W - 1], P[c - W], P[c - W + 1], P[c - 1], P[c], P[c + 1],
-                                 P[c + W - 1], P[c + W], P[c + W + 1], Dl[c - W - 1], Dl[c - W],
-                                 Dl[c - W + 1], Dl[c - 1], Dl[c], Dl[c + 1], Dl[c + W - 1],
-                                 Dl[c + W], Dl[c + W + 1], Tf);
-}
-
 template <typename T>
 __host__ __device__ inline int lut_slots(int ncls) {
     int n = ncls * K_N;
@@ -146,7 +136,8 @@ __host__ __device__ inline size_t tile_wind_elems(int TX, int TY, int ky) {
 // more FP64 than the right-hand side); otherwise per node and stage.  Small
 // meshes, where this kernel is the default, are bound by the latency of its
 // chain of stages.  Measured, us per step (GB300), before and now: 100^2 nodes
-// in FP64 53.7 and 30.0 (25.7 with the tables formed during the step before).
+// in FP64 53.7 and 24.3 (30.0 with the steps not chained, see launch_chained,
+// and the quadrature of a node by one lane).
 // ---------------------------------------------------------------------------
 template <typename T, bool TAB>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 : kTileCtasPerSmF32)
@@ -384,21 +375,30 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 :
 
     // ---- G: fuel fraction on the tile, heat contributions dF * H per node
     T *Q = P0;  // P0/P1 are dead: 2 values per tile node
-    for (int e = tid; e < TX * TY; e += kThreads) {
+    // a node's four subcells by two lanes, the lower two and the upper two,
+    // where the tile's threads suffice: the quadrature is the longest chain of
+    // the kernel.  (100^2 nodes in FP64 with a fire, tiles of 100 nodes: 25.7 us
+    // per step by one lane, 24.3 by two; 370x290 in FP32, tiles of 200 nodes:
+    // 2 % slower by two.)
+    const int lanes = 2 * TX * TY <= kThreads && a.scheme != 1 ? 2 : 1;
+    for (int e0 = 0; e0 < lanes * TX * TY; e0 += kThreads) {
+        const int e = lanes == 2 ? (e0 + tid) >> 1 : e0 + tid, side = lanes == 2 ? tid & 1 : 0;
         int lx, ly;
         split(e, TX, lx, ly);
-        const int gy = y0 + ly;
-        T hs = T(0), hq = T(0);
-        if (lx < TXa && ly < TYa) {
-            const int gx = x0 + lx;
-            const size_t g = WF_CHK((size_t)gy * nx + gx, (long long)nx * ny, st);
-            const T Fo = F_in[g];
+        const int gy = y0 + ly, gx = x0 + lx;
+        const bool in = e < TX * TY && lx < TXa && ly < TYa;
+        const size_t g = in ? WF_CHK((size_t)gy * nx + gx, (long long)nx * ny, st) : 0;
+        const int cc = (ly + 1) * BW1 + (lx + 1);
+        T Fo = T(0), Fn = T(1);
+        const T *co = lut;
+        if (in) {
+            Fo = F_in[g];
             int cls = fuel[g];
             cls = cls > ncm1 ? ncm1 : cls;
-            const T *co = lut + cls * K_N;
-            const int cc = (ly + 1) * BW1 + (lx + 1);
-            T Fn;
-            if (a.scheme == 1) {
+            co = lut + cls * K_N;
+        }
+        if (a.scheme == 1) {
+            if (in) {
                 T p9[9], d9[9];
 #pragma unroll
                 for (int b = 0; b < 3; ++b)
@@ -408,9 +408,21 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 :
                         d9[b * 3 + h] = Dl[cc + (b - 1) * BW1 + (h - 1)];
                     }
                 Fn = cell_fraction_linear_vals<T>(p9, d9, co[K_TF]);
-            } else {
-                Fn = cell_fraction<T>(P2, Dl, cc, BW1, co[K_TF]);
             }
+        } else {
+            T bW = T(0), bE = T(0), uW = T(0), uE = T(0);
+            if (in) cell_fraction_half<T>(P2, Dl, cc, BW1, side, co[K_TF], bW, bE);
+            if (lanes == 2) {
+                uW = __shfl_down_sync(0xffffffffu, bW, 1);
+                uE = __shfl_down_sync(0xffffffffu, bE, 1);
+            } else if (in) {
+                cell_fraction_half<T>(P2, Dl, cc, BW1, 1, co[K_TF], uW, uE);
+            }
+            Fn = fma(T(-0.25), ((bW + bE) + uW) + uE, T(1));
+        }
+        if (side || e >= TX * TY) continue;
+        T hs = T(0), hq = T(0);
+        if (in) {
             F_out[g] = Fn;
             const T dF = Fo - Fn;
             hs = dF * (nhs ? nhs[g] : co[K_HS]);
