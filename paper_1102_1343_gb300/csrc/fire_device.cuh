@@ -167,9 +167,6 @@ __device__ __forceinline__ bool any_sign(float a, float b, float c) {
 }
 __device__ __forceinline__ bool nonzero(float x) { return x != 0.0f; }
 __device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
-// a number below 0 among three (FP64: a set sign)
-__device__ __forceinline__ bool any_neg(float a, float b, float c) { return fminf(fminf(a, b), c) < 0.0f; }
-__device__ __forceinline__ bool any_neg(double a, double b, double c) { return any_sign(a, b, c); }
 // x <= 0
 __device__ __forceinline__ bool le0(float x) { return x <= 0.0f; }
 __device__ __forceinline__ bool le0(double x) { return __double_as_longlong(x) <= 0; }
@@ -342,7 +339,7 @@ __device__ __forceinline__ T cell_fraction_vals(T p00, T p01, T p02, T p10, T p1
 
 // The burned fractions of the two subcells below (side 0) or above (side 1) the
 // cell's centre row, west then east, with the operations of
-// cell_fraction_vals: node c of P and D (rows S apart), zeros where the
+// cell_fraction_vals (FP64): node c of P and D (rows S apart), zeros where the
 // neighbourhood has no burning node.
 template <typename T>
 __device__ __forceinline__ void cell_fraction_half(const T *P, const T *D, int c, int S, int side, T Tf,
@@ -350,7 +347,7 @@ __device__ __forceinline__ void cell_fraction_half(const T *P, const T *D, int c
     bW = bE = T(0);
     const int o = side ? c + S : c - S, x = side ? c - S : c + S;  // this side's row, the other
     const T o0 = P[o - 1], o1 = P[o], o2 = P[o + 1], m0 = P[c - 1], m1 = P[c], m2 = P[c + 1];
-    if (!any_neg(o0, o1, o2) && !any_neg(m0, m1, m2) && !any_neg(P[x - 1], P[x], P[x + 1])) return;
+    if (!any_sign(o0, o1, o2) && !any_sign(m0, m1, m2) && !any_sign(P[x - 1], P[x], P[x + 1])) return;
     const T e0 = D[o - 1], e1 = D[o], e2 = D[o + 1], f0 = D[c - 1], f1 = D[c], f2 = D[c + 1];
     const T h = T(0.5), q = T(0.25);
     T pW = h * (m0 + m1), pE = h * (m1 + m2), pO = h * (o1 + m1);

@@ -99,6 +99,16 @@ __device__ void fill_ghosts_pd(T *P, T *Dl, int BW, int BH, int ox, int oy, int 
     __syncthreads();
 }
 
+// Fuel fraction of the cell at index c of the staged psi^{n+1} (P) and
+// Dl = t - t_i (row pitch W).
+template <typename T>
+__device__ __forceinline__ T cell_fraction(const T *P, const T *Dl, int c, int W, T Tf) {
+    return cell_fraction_vals<T>(P[c - W - 1], P[c - W], P[c - W + 1], P[c - 1], P[c], P[c + 1],
+                                 P[c + W - 1], P[c + W], P[c + W + 1], Dl[c - W - 1], Dl[c - W],
+                                 Dl[c - W + 1], Dl[c - 1], Dl[c], Dl[c + 1], Dl[c + W - 1],
+                                 Dl[c + W], Dl[c + W + 1], Tf);
+}
+
 template <typename T>
 __host__ __device__ inline int lut_slots(int ncls) {
     int n = ncls * K_N;
@@ -375,12 +385,13 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 :
 
     // ---- G: fuel fraction on the tile, heat contributions dF * H per node
     T *Q = P0;  // P0/P1 are dead: 2 values per tile node
-    // a node's four subcells by two lanes, the lower two and the upper two,
-    // where the tile's threads suffice: the quadrature is the longest chain of
-    // the kernel.  (100^2 nodes in FP64 with a fire, tiles of 100 nodes: 25.7 us
-    // per step by one lane, 24.3 by two; 370x290 in FP32, tiles of 200 nodes:
-    // 2 % slower by two.)
-    const int lanes = 2 * TX * TY <= kThreads && a.scheme != 1 ? 2 : 1;
+    // FP64: a node's four subcells by two lanes, the lower two and the upper
+    // two, where the tile's threads suffice: the quadrature is the longest chain
+    // of the kernel (100^2 nodes with a fire, tiles of 100 nodes: 25.7 us per
+    // step by one lane, 24.3 by two; tiles of 200 nodes 2 % slower by two).  In
+    // FP32 the chain is short, and the sum of the four keeps the form (and the
+    // rounding) that the other kernels give it.
+    const int lanes = sizeof(T) == 8 && 2 * TX * TY <= kThreads && a.scheme != 1 ? 2 : 1;
     for (int e0 = 0; e0 < lanes * TX * TY; e0 += kThreads) {
         const int e = lanes == 2 ? (e0 + tid) >> 1 : e0 + tid, side = lanes == 2 ? tid & 1 : 0;
         int lx, ly;
@@ -409,7 +420,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 :
                     }
                 Fn = cell_fraction_linear_vals<T>(p9, d9, co[K_TF]);
             }
-        } else {
+        } else if constexpr (sizeof(T) == 8) {
             T bW = T(0), bE = T(0), uW = T(0), uE = T(0);
             if (in) cell_fraction_half<T>(P2, Dl, cc, BW1, side, co[K_TF], bW, bE);
             if (lanes == 2) {
@@ -418,7 +429,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 :
             } else if (in) {
                 cell_fraction_half<T>(P2, Dl, cc, BW1, 1, co[K_TF], uW, uE);
             }
-            Fn = fma(T(-0.25), ((bW + bE) + uW) + uE, T(1));
+            // (added without contraction: the same bits by one lane and by two)
+            Fn = fma(T(-0.25), __dadd_rn(__dadd_rn(__dadd_rn(bW, bE), uW), uE), T(1));
+        } else {
+            if (in) Fn = cell_fraction<T>(P2, Dl, cc, BW1, co[K_TF]);
         }
         if (side || e >= TX * TY) continue;
         T hs = T(0), hq = T(0);
