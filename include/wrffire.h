@@ -446,9 +446,9 @@ int fire_kernel_time_ms(fire_ctx *ctx, double *ms, long *launches);
  *   cuda_stream               stream for all work of the call
  * Ignitions are not applied: the state passed in already holds them.
  * Fuel classes are checked as fire_init checks them (FIRE_ERR_ARG).
- * Intermediate values (the class table, its coefficients, the start and end
+ * Intermediate values (the coefficients of the classes, the start and end
  * time, and the status word when status_dev is NULL) live in one file-scope
- * device array of about 11 KB per device, held until the process exits.
+ * device array of about 5 KB per device, held until the process exits.
  * The first call on a device looks up that array's device address
  * (cudaGetSymbolAddress) with the device current; make it before any stream
  * capture.  Every call shares the array and it keeps the last call's

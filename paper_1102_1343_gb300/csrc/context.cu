@@ -80,10 +80,9 @@ struct fire_ctx {
     long launches = 0;
     double ms_done = 0;
 
-    // adaptive choice between the FP32 warp kernels (bitwise equal results):
-    // the default strips on a nearly unburnt mesh, the dense variant with
-    // shorter strips once enough of it burns; on while the context runs
-    // fire_init's default warp strips
+    // adaptive choice between the two names of the FP32 row kernel: the default
+    // strips on a nearly unburnt mesh, the dense variant with shorter strips once
+    // enough of it burns; on while the context runs fire_init's default strips
     bool adaptive = false;
     bool ad_dense = false;                       // the dense variant is chosen
     int ad_kx = 0, ad_ky = 0, ad_dense_ky = 0;   // the two shapes
@@ -419,9 +418,8 @@ int default_kernel(fire_ctx *c) {
 }
 
 // burnt fraction at which the dense variant takes over, and below which the
-// default strips come back; measured on the 8200x8200 mesh: the default
-// strips are 6-10 % faster on a nearly unburnt mesh, the dense 6x6 strips
-// 1 % faster at 0.6 % burnt and 11-15 % faster from 2 % burnt on
+// default strips come back (both names are the row kernel now, launched with
+// the rows of warp_launch_rows: the choice changes no time of a default context)
 constexpr double kAdaptOn = 0.005, kAdaptOff = 0.0025;
 constexpr long kAdaptEvery = 64;  // steps between counts
 
