@@ -342,13 +342,14 @@ int ens_plan(fire_ensemble *e) {
     }
     {
         // the limit is a property of the kernel function on a device, shared by
-        // all ensembles there
+        // all ensembles there: one slot per function (the parity of the mesh
+        // widths selects one in the warp form alone)
         static std::mutex mu;
         static size_t current[kMaxDevices][16] = {};
         std::lock_guard<std::mutex> lock(mu);
         const int dev = attr_device();
-        const int form = (f64 ? 1 : 0) + (e->variant == FIRE_KERNEL_WARP ? 2 : 0) + (e->nc ? 4 : 0) +
-                         (e->even ? 8 : 0);
+        const bool warp = e->variant == FIRE_KERNEL_WARP;
+        const int form = (f64 ? 1 : 0) + (warp ? 2 : 0) + (e->nc ? 4 : 0) + (warp && e->even ? 8 : 0);
         if (dev < 0 || smem > current[dev][form]) {
             ENS_CHECK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             if (dev >= 0) current[dev][form] = smem;
