@@ -906,9 +906,12 @@ __global__ void __launch_bounds__(32 * kRowWarps, (row_ctas<T, MODE>())) k_fire_
     RowSmem<T, NW> sm;
     sm.carve(row_smem, a.ky, a.sry, a.ncls);
     const double tstart = *a.t_in;
-    if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0) *a.t_out = tstart + a.dt;
+    const int band = blockIdx.z * gridDim.y + blockIdx.y;  // (z: beyond 65535 rows of strips)
+    const int y0 = band * a.ky * a.sry;
+    if (y0 >= a.ny) return;
+    if (threadIdx.x == 0 && blockIdx.x == 0 && band == 0) *a.t_out = tstart + a.dt;
     RowStrip<T, MODE, NW, WIDTH, FULL> s(a, sm, row_smem);
-    s.run(blockIdx.x * a.kx * a.srx, blockIdx.y * a.ky * a.sry, tstart);
+    s.run(blockIdx.x * a.kx * a.srx, y0, tstart);
     const int stw = __reduce_or_sync(0xffffffffu, s.st);
     if ((threadIdx.x & 31) == 0 && stw) atomicOr(a.status, stw);
 }
@@ -961,7 +964,8 @@ cudaError_t launch_warp(const StepArgs &args, cudaStream_t s) {
         return cudaErrorInvalidValue;
     a.ky = row_strip_bands(a.ky, a.sry);
     const int L = a.ky * a.sry;
-    dim3 grid((a.nx + W - 1) / W, (a.ny + L - 1) / L);
+    const unsigned bands = (a.ny + L - 1) / L, rows = bands < 65535u ? bands : 65535u;
+    const dim3 grid((a.nx + W - 1) / W, rows, (bands + rows - 1) / rows);
     const size_t smem = warp_smem_bytes<T>(a.ky, a.sry, a.ncls);
     const int mode = a.nco[0] ? ROW_NC : a.mult ? ROW_MULT : ROW_PLAIN;
     const bool even = (a.nx & 1) == 0, full = a.F_out != nullptr;
