@@ -1385,11 +1385,8 @@ constexpr int kMisfitBlocks = 304;
 int cuda_fail(cudaError_t e, const char *where) {
     if (e == cudaSuccess) return FIRE_OK;
     record_cuda_error(e, where);
-    if (e == cudaErrorMemoryAllocation) {
-        cudaGetLastError();
-        return FIRE_ERR_OOM;
-    }
-    return FIRE_ERR_CUDA;
+    cudaGetLastError();  // reported here: the next call starts without it
+    return e == cudaErrorMemoryAllocation ? FIRE_ERR_OOM : FIRE_ERR_CUDA;
 }
 #define ADJ_CHECK(call)                                   \
     do {                                                  \

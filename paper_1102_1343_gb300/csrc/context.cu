@@ -126,11 +126,8 @@ namespace {
 int cuda_err_at(cudaError_t e, const char *where) {
     if (e == cudaSuccess) return FIRE_OK;
     record_cuda_error(e, where);
-    if (e == cudaErrorMemoryAllocation) {
-        cudaGetLastError();
-        return FIRE_ERR_OOM;
-    }
-    return FIRE_ERR_CUDA;
+    cudaGetLastError();  // reported here: the next call starts without it
+    return e == cudaErrorMemoryAllocation ? FIRE_ERR_OOM : FIRE_ERR_CUDA;
 }
 
 #define cuda_err(call) cuda_err_at((call), #call)

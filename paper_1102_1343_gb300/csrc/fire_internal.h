@@ -105,7 +105,9 @@ cudaError_t launch_chained(bool chained, void (*kernel)(P...), dim3 grid, dim3 b
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = chained ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+    if (e != cudaSuccess) cudaGetLastError();  // (the caller reports it; the next call starts without)
+    return e;
 }
 
 struct IgnSeg {
