@@ -234,7 +234,7 @@ __device__ __forceinline__ void node_partials(T p, T pl, T pr, T pd, T pu, T idx
         cx *= i2dx;
         cy *= i2dy;
         const T cn2 = fma(cx, cx, cy * cy);
-        normal = __double2hiint(cn2) >= 0x00200000;
+        normal = normal64(cn2);
         if (normal) rc = rsqrt64(cn2);
         nxv = cx * rc;
         nyv = cy * rc;
@@ -266,7 +266,7 @@ __device__ __forceinline__ void node_partials(T p, T pl, T pr, T pd, T pu, T idx
     const T tpp = pos_val(tp);
     const T pwv = Mth<T>::pw(Ue, e.co[K_B]);
     const T inner = e.co[K_R0] + e.co[K_C] * pwv + e.co[K_D] * tpp * tpp;
-    const bool active = gt_nn(inner, e.co[K_S0]);
+    const bool active = gt_nn(pos_val(inner), e.co[K_S0]);
     const T St = active ? inner : e.co[K_S0];
     const T S = e.m * St;
     const T lap = (dxp - dxm) + (dyp - dym);

@@ -134,7 +134,7 @@ struct Mth<double> {
     // norm, two products); zero vector when the norm vanishes
     static __device__ __forceinline__ void unit(double cx, double cy, double &nx, double &ny) {
         const double n2 = fma(cx, cx, cy * cy);
-        if (__double2hiint(n2) >= 0x00200000) {
+        if (normal64(n2)) {
             const double r = rsqrt64(n2);
             nx = cx * r;
             ny = cy * r;
@@ -158,18 +158,24 @@ __device__ __forceinline__ bool finite_val(double x) {
     return (__double_as_longlong(x) & 0x7ff0000000000000LL) != 0x7ff0000000000000LL;
 }
 
-// a set sign among three numbers (FP64: no instruction of the narrow pipe)
+// a number with a set sign among three (FP64: no instruction of the narrow pipe;
+// NaN, a quiet one, is none)
 __device__ __forceinline__ bool any_sign(double a, double b, double c) {
-    return (__double2hiint(a) | __double2hiint(b) | __double2hiint(c)) < 0;
+    const unsigned s = 0x80000000u;
+    return min(min((unsigned)__double2hiint(a) ^ s, (unsigned)__double2hiint(b) ^ s),
+               (unsigned)__double2hiint(c) ^ s) <= 0x7ff00000u;
 }
 __device__ __forceinline__ bool any_sign(float a, float b, float c) {
-    return (__float_as_int(a) | __float_as_int(b) | __float_as_int(c)) < 0;
+    return fminf(fminf(a, b), c) < 0.0f;
 }
 __device__ __forceinline__ bool nonzero(float x) { return x != 0.0f; }
 __device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
 // x <= 0
 __device__ __forceinline__ bool le0(float x) { return x <= 0.0f; }
-__device__ __forceinline__ bool le0(double x) { return __double_as_longlong(x) <= 0; }
+__device__ __forceinline__ bool le0(double x) {
+    const long long b = __double_as_longlong(x);
+    return b <= 0 && (unsigned long long)b <= 0xfff0000000000000ull;
+}
 
 // extrapolated ghost value beyond the last node p0 (p1 the one before it),
 // Sect. 3.1: max{p0 + (p0 - p1), p0, p1}

@@ -17,20 +17,29 @@
 
 namespace wf {
 
-// max{x, 0} (a NaN with a clear sign stays)
+// The tests below are those of the comparisons that they stand for, with NaN
+// counted as there: not above 0, not at most 0.  (Where only the upper word is
+// looked at, x is the result of an operation and a NaN a quiet one.)
+
+// x > 0 ? x : 0
 __device__ __forceinline__ double pos64(double x) {
-    const int hi = __double2hiint(x), m = ~(hi >> 31);
-    return __hiloint2double(hi & m, __double2loint(x) & m);
+    return (unsigned)__double2hiint(x) <= 0x7ff00000u ? x : 0.0;
 }
-// the larger and the smaller of two numbers that are not negative
+// the larger and the smaller of two numbers that are neither negative nor NaN
 __device__ __forceinline__ double max_nn(double a, double b) {
     return (unsigned long long)__double_as_longlong(a) > (unsigned long long)__double_as_longlong(b) ? a : b;
 }
 __device__ __forceinline__ double min_nn(double a, double b) {
     return (unsigned long long)__double_as_longlong(a) < (unsigned long long)__double_as_longlong(b) ? a : b;
 }
-// x > 0 (a NaN with a clear sign too)
-__device__ __forceinline__ bool gt0(double x) { return __double_as_longlong(x) > 0; }
+// x > 0
+__device__ __forceinline__ bool gt0(double x) {
+    return (unsigned long long)__double_as_longlong(x) - 1 < 0x7ff0000000000000ull;
+}
+// x at least 2^-1021 and finite
+__device__ __forceinline__ bool normal64(double x) {
+    return (unsigned)__double2hiint(x) - 0x00200000u < 0x7fd00000u;
+}
 
 // One step of third order from the hardware's coarse approximation y of
 // 1/sqrt(x) (relative error below 2^-20): with e = 1 - x y^2 the value is
@@ -47,7 +56,7 @@ __device__ __forceinline__ double rsqrt64(double x) {
 }
 // sqrt of x >= 0: with t = x y the value is t (1 - e)^(-1/2), e = 1 - t y
 __device__ __forceinline__ double sqrt64(double x) {
-    if ((unsigned)__double2hiint(x) - 0x00200000u >= 0x7fd00000u) return sqrt(x);  // 0, subnormal, inf, NaN
+    if (!normal64(x)) return sqrt(x);  // 0, subnormal, inf, NaN
     const double y = rsqrt_seed(x), t = x * y, e = fma(-t, y, 1.0);
     return fma(t * e, fma(0.375, e, 0.5), t);
 }
@@ -140,10 +149,11 @@ __device__ __forceinline__ double neg_rhs64(double p, double pl, double pr, doub
     const double gx = max_nn(pos64(xm), pos64(xp)), gy = max_nn(pos64(ym), pos64(yp));
     const double grad = sqrt64(fma(gx, gx, gy * gy));
     const double n2 = fma(cx, cx, cy * cy);
-    const double rn = __double2hiint(n2) < 0x00200000 ? 0.0 : rsqrt64(n2);
+    const double rn = normal64(n2) ? rsqrt64(n2) : 0.0;
     const double U = fma(un, cx, vn * cy) * rn, tp = pos64(fma(zx, cx, zy * cy) * rn);
     const double pw = wind_power64(min_nn(pos64(U), e), b);
-    const double s = max_nn(fma(d * tp, tp, fma(c, pw, R0)), S0);
+    // (R0 and c are negative for a moisture or a heat content without sense)
+    const double s = max_nn(pos64(fma(d * tp, tp, fma(c, pw, R0))), S0);
     double S = HASM ? m * s : s;
     if (iso) S *= idx;
     const double nlap = (xm + xp) + (ym + yp);
