@@ -120,11 +120,7 @@ struct Mth<double> {
     static __device__ __forceinline__ double pw(double x, double b) { return wind_power64(x, b); }
     static __device__ __forceinline__ double ex(double x) { return exp(x); }
     static __device__ __forceinline__ double rcp(double x) { return rcp64(x); }
-    // a/b for a normal b: the quotient by the reciprocal, corrected once
-    static __device__ __forceinline__ double dv(double a, double b) {
-        const double y = rcp64(b), q = a * y;
-        return fma(fma(-b, q, a), y, q);
-    }
+    static __device__ __forceinline__ double dv(double a, double b) { return div64(a, b); }
     static __device__ __forceinline__ double one_minus_div(double a, double b) {
         return 1.0 - a / b;
     }

@@ -41,10 +41,12 @@ __device__ __forceinline__ bool normal64(double x) {
     return (unsigned)__double2hiint(x) - 0x00200000u < 0x7fd00000u;
 }
 
-// One step of third order from the hardware's coarse approximation y of
-// 1/sqrt(x) (relative error below 2^-20): with e = 1 - x y^2 the value is
-// y (1 - e)^(-1/2) = y (1 + e/2 + 3/8 e^2 + ...), and what is left out is below
-// 2^-60.  x is normal and finite.
+// Roots and reciprocals by Householder's iteration (A. S. Householder, The
+// Numerical Treatment of a Single Nonlinear Equation, 1970), one step of third
+// order from the hardware's coarse approximation y (relative error below
+// 2^-20).  1/sqrt(x): with e = 1 - x y^2 the value is y (1 - e)^(-1/2) =
+// y (1 + e/2 + 3/8 e^2 + ...), what is left out is below 2^-58 and the error
+// below 1.6 times 2^-53.  x is normal64.
 __device__ __forceinline__ double rsqrt_seed(double x) {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
@@ -60,8 +62,8 @@ __device__ __forceinline__ double sqrt64(double x) {
     const double y = rsqrt_seed(x), t = x * y, e = fma(-t, y, 1.0);
     return fma(t * e, fma(0.375, e, 0.5), t);
 }
-// 1/x of a normal finite x: the hardware's approximation and a step of third
-// order, 1/x = y/(1 - e) with e = 1 - x y
+// 1/x, 2^-1021 <= |x| < 2^1022 (a normal reciprocal): with e = 1 - x y the value
+// is y/(1 - e) = y (1 + e + e^2 + ...); the error is below 1.1 times 2^-53
 __device__ __forceinline__ double rcp64(double x) {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
@@ -107,11 +109,18 @@ __device__ __forceinline__ double pow64(double x, double b) {
     const double v = fma(T, p * f, T);
     return __hiloint2double(__double2hiint(v) + ((j >> 7) << 20), __double2loint(v));
 }
-// the capped wind component's power: 0 where it is 0 (or its power beyond the
-// range of doubles)
+// a/b by the reciprocal and one correction with the exact residual (P. W.
+// Markstein, IBM J. Res. Dev. 34 (1990) 111); divisors that have no normal
+// reciprocal take the ordinary quotient
+__device__ __forceinline__ double div64(double a, double b) {
+    if (((unsigned)__double2hiint(b) & 0x7fffffffu) - 0x00200000u >= 0x7fb00000u) return a / b;
+    const double y = rcp64(b), q = a * y;
+    return fma(fma(-b, q, a), y, q);
+}
+// x^b of the capped wind component x >= 0: 0 where it is 0
 __device__ __forceinline__ double wind_power64(double x, double b) {
+    if (__double_as_longlong(x) == 0) return 0.0;
     const int hi = __double2hiint(x);
-    if (hi < 0x00200000) return 0.0;
     // |b log2 x| < 900: x in [2^-64, 2^64) and b < 14 without a closer look
     if ((unsigned)(hi - 0x3bf00000) < 0x08000000u && __double2hiint(b) < 0x402c0000) return pow64(x, b);
     return exp2(b * log2(x));

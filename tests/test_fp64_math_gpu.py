@@ -7,8 +7,10 @@ it enters, 0.5 u) and what the series leaves out (2^-7 u), so 1.6 u.  rcp64 and
 the quotient: the last rounding and a residual below 2^-6 u, so 1.1 u.  The
 power: y = b log2 x is rounded once (|y| u, times ln 2), the table, its product
 and the last sum 3 u more.  Outside its fast range it is exp2(b log2 x) of the
-CUDA functions: three roundings of y (each to 1.5 u) and 3 u."""
+CUDA functions: three roundings of y (each to 1.5 u) and 3 u.  And the adjoint's quotient by a capped wind component
+below the normal range."""
 import ctypes as C
+import dataclasses
 import os
 import subprocess
 
@@ -95,3 +97,29 @@ def test_power(probe):
         got = probe(POW, x, np.full_like(x, b)).astype(np.longdouble)
         assert (np.abs(got - want) <= want * U * (3.2 * np.abs(y) + 3) + 5e-324).all(), b
     assert (probe(POW, np.zeros(3), np.array([0.5, 1.0, 2.0])) == 0).all()
+
+
+def test_wind_below_the_normal_range():
+    """Capped wind components between 0 and the smallest normal number: the
+    gradients are the oracle's (the quotient by such a component)."""
+    import oracle
+    import paper_1102_1343_gb300 as pkg
+    from paper_1102_1343_gb300 import build, synth
+    build.build()
+    w = synth.random_landscape(8, 7, sr=10, dx_atm=60.0, seed=9, ignition="center", steps=6, dt=0.5)
+    w = dataclasses.replace(w, classes=[synth.nominal_class(fgi=0.5)], fuel=np.zeros((70, 80), np.uint8))
+    w = dataclasses.replace(w, ignitions=[synth.point_ignition(240.0, 210.0, radius=20.0)], mult=np.full((70, 80), 40.0),
+                            u=w.u * 1e-310, v=w.v * 1e-310)
+    y, x = np.indices((70, 80))
+    tobs = np.where((x - 40) ** 2 + (y - 35) ** 2 < 400, 2.0, np.nan)
+    Jr, *ref = oracle.OracleFire.from_workload(w).adjoint(w.u, w.v, w.dt, w.steps, tobs)
+    m = pkg.FireModel.from_workload(w, precision="fp64")
+    u, v = m.wind(w.u, w.v)
+    J, *g = m.adjoint(u, v, w.dt, w.steps, tobs, ckpt_every=2)
+    assert np.abs(ref[0]).max() > 0 and abs(J - Jr) <= 1e-10 * Jr
+    for a, b in zip(g[:2], ref[:2]):
+        a = a.cpu().numpy()
+        assert np.isfinite(a).all() and np.linalg.norm(a - b) <= 1e-8 * np.linalg.norm(b)
+    for a in g[2:]:
+        assert np.isfinite(a.cpu().numpy()).all()
+    m.close()
