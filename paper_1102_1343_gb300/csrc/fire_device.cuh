@@ -161,9 +161,6 @@ __device__ __forceinline__ bool any_sign(double a, double b, double c) {
     return min(min((unsigned)__double2hiint(a) ^ s, (unsigned)__double2hiint(b) ^ s),
                (unsigned)__double2hiint(c) ^ s) <= 0x7ff00000u;
 }
-__device__ __forceinline__ bool any_sign(float a, float b, float c) {
-    return fminf(fminf(a, b), c) < 0.0f;
-}
 __device__ __forceinline__ bool nonzero(float x) { return x != 0.0f; }
 __device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
 // x <= 0

@@ -418,9 +418,20 @@ struct MarchStrip {
                     p[b][3] = sm.SQ[sl[b] * NT + c + 1].x;
                 }
             }
-            // (a set sign: psi < 0 or -0, for which the quadrature gives 1 too)
-            const bool burning = any_sign(p[0][0], p[1][0], p[2][0]) || any_sign(p[0][1], p[1][1], p[2][1]) ||
-                                 any_sign(p[0][2], p[1][2], p[2][2]) || any_sign(p[0][3], p[1][3], p[2][3]);
+            // FP64: by a set sign, psi < 0 or -0, for which the quadrature gives
+            // 1 too (FP32 by minima: 1000^2 nodes, 12 steps, 1.64 ms, and 1.72
+            // by the signs)
+            bool burning;
+            if constexpr (sizeof(T) == 8) {
+                burning = any_sign(p[0][0], p[1][0], p[2][0]) || any_sign(p[0][1], p[1][1], p[2][1]) ||
+                          any_sign(p[0][2], p[1][2], p[2][2]) || any_sign(p[0][3], p[1][3], p[2][3]);
+            } else {
+                T vmin[4];
+#pragma unroll
+                for (int h = 0; h < 4; ++h) vmin[h] = min_val(min_val(p[0][h], p[1][h]), p[2][h]);
+                const T mid = min_val(vmin[1], vmin[2]);
+                burning = min_val(vmin[0], mid) < T(0) || min_val(mid, vmin[3]) < T(0);
+            }
             const bool edge = xa <= 0 || xa + 1 >= nx - 1 || rd == 0 || rd == ny - 1;
             T Fn[2] = {T(1), T(1)};
             if (burning || edge) {

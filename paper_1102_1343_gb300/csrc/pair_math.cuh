@@ -60,15 +60,19 @@ __device__ __forceinline__ float max3_val(float a, float b, float c) {
 __device__ __forceinline__ double max3_val(double a, double b, double c) { return fmax(fmax(a, b), c); }
 
 // unit vectors of two (cx, cy): Mth::unit on pairs
+template <bool ROW>
 __device__ __forceinline__ void unit2(float2 cx, float2 cy, float2 &nx, float2 &ny) {
     // 2^63 = 1/sqrt(kNormMin): where both components vanish the vector stays
     // zero (0 times that)
     const float2 n2 = fma2(cx, cx, mul2(cy, cy));
-    const float2 r = make_float2(fminf(rsqrt_ftz(n2.x), 9223372036854775808.0f),
-                                 fminf(rsqrt_ftz(n2.y), 9223372036854775808.0f));
+    const float2 r = ROW ? make_float2(fminf(rsqrt_ftz(n2.x), 9223372036854775808.0f),
+                                       fminf(rsqrt_ftz(n2.y), 9223372036854775808.0f))
+                         : make_float2(rsqrt_ftz(fmaxf(n2.x, Mth<float>::kNormMin)),
+                                       rsqrt_ftz(fmaxf(n2.y, Mth<float>::kNormMin)));
     nx = mul2(cx, r);
     ny = mul2(cy, r);
 }
+template <bool ROW>
 __device__ __forceinline__ void unit2(double2 cx, double2 cy, double2 &nx, double2 &ny) {
     Mth<double>::unit(cx.x, cy.x, nx.x, ny.x);
     Mth<double>::unit(cx.y, cy.y, nx.y, ny.y);
@@ -99,8 +103,11 @@ struct WCoef {
 // Godunov's |D| = max(D-, -D+, 0) and the Laplacian -(D-x + (-D+x)) - (...)
 // need no negated operand, and G = S (|grad psi| - eps Lap) =
 // S (|grad psi| + eps (D-x - D+x + D-y - D+y)).
-// HASM false: every multiplier is 1 (m is not read).
-template <typename T, bool HASM = true>
+// HASM false: every multiplier is 1 (m is not read).  ROW: the forms of the row
+// kernel, with a few products packed and the normal's limit after the root: the
+// same bits, fewer instructions there, but registers spilled in the marching
+// strips, which have none left.
+template <typename T, bool HASM = true, bool ROW = false>
 __device__ __forceinline__ typename PairT<T>::t neg_rhs2(
     typename PairT<T>::t p, typename PairT<T>::t pl, typename PairT<T>::t pr,
     typename PairT<T>::t pd, typename PairT<T>::t pu, typename PairT<T>::t idx2,
@@ -128,16 +135,18 @@ __device__ __forceinline__ typename PairT<T>::t neg_rhs2(
     const V g2 = fma2(gx, gx, mul2(gy, gy));
     // central differences, zeroed at the rounding level of their values
     V ddx = sub2(pr, pl), ddy = sub2(pu, pd);
-    const V z = splat<V>(Mth<T>::kGradZero);
-    const V zx2 = mul2(z, mk2(abs_val(pr.x) + abs_val(pl.x), abs_val(pr.y) + abs_val(pl.y)));
-    const V zy2 = mul2(z, mk2(abs_val(pu.x) + abs_val(pd.x), abs_val(pu.y) + abs_val(pd.y)));
+    const T z = Mth<T>::kGradZero;
+    const V ax = mk2(abs_val(pr.x) + abs_val(pl.x), abs_val(pr.y) + abs_val(pl.y));
+    const V ay = mk2(abs_val(pu.x) + abs_val(pd.x), abs_val(pu.y) + abs_val(pd.y));
+    const V zx2 = ROW ? mul2(splat<V>(z), ax) : mk2(z * ax.x, z * ax.y);
+    const V zy2 = ROW ? mul2(splat<V>(z), ay) : mk2(z * ay.x, z * ay.y);
     ddx.x = abs_val(ddx.x) <= zx2.x ? T(0) : ddx.x;
     ddx.y = abs_val(ddx.y) <= zx2.y ? T(0) : ddx.y;
     ddy.x = abs_val(ddy.x) <= zy2.x ? T(0) : ddy.x;
     ddy.y = abs_val(ddy.y) <= zy2.y ? T(0) : ddy.y;
     const V cx = mul2(ddx, i2dx2), cy = mul2(ddy, i2dy2);
     V nxv, nyv;
-    unit2(cx, cy, nxv, nyv);
+    unit2<ROW>(cx, cy, nxv, nyv);
     const V U = fma2(un, nxv, mul2(vn, nyv));
     const V tp = fma2(zx, nxv, mul2(zy, nyv));
     // spread rate, eq. (spread-WRF-Fire)
@@ -146,7 +155,8 @@ __device__ __forceinline__ typename PairT<T>::t neg_rhs2(
     Ue.y = min_val(max_val(U.y, T(0)), co.e.y);
     tq.x = max_val(tp.x, T(0));
     tq.y = max_val(tp.y, T(0));
-    pw = pow_pair(Ue, co.b);
+    if constexpr (ROW) pw = pow_pair(Ue, co.b);
+    else pw = mk2(Mth<T>::pw(Ue.x, co.b.x), Mth<T>::pw(Ue.y, co.b.y));
     V s = fma2(mul2(co.d, tq), tq, fma2(co.c, pw, co.R0));
     s.x = max_val(s.x, co.S0.x);
     s.y = max_val(s.y, co.S0.y);

@@ -46,7 +46,10 @@ struct W4Env {  // environment of a row: what stage 2 reuses from stage 1
     float2 R0[2], cc[2], dd[2];  // per-node coefficients (NC only)
 };
 
-template <bool NC>
+// MANY: strips of more than 32 atmospheric cells (refinements 1 to 3).  (The loop
+// over them costs the others registers: 1000^2 nodes, 12 steps, 2.97 ms without it
+// and 3.02 with.)
+template <bool NC, bool MANY>
 struct WarpStrip4 {
     using V = float2;
     const StepArgs &a;
@@ -598,7 +601,7 @@ struct WarpStrip4 {
                 make_float4(acc_q[0].x, acc_q[0].y, acc_q[1].x, acc_q[1].y);
             __syncwarp();
             const int cells = Wa / srx;
-            for (int c = lane; c * srx < Wa; c += 32) {  // one lane per atmospheric cell
+            for (int c = lane; c < cells; c += 32) {  // one lane per atmospheric cell
                 float h0 = 0.0f, h1 = 0.0f;
                 for (int e = 0; e < srx; ++e) {
                     const int lc = 4 + c * srx + e;
@@ -608,6 +611,7 @@ struct WarpStrip4 {
                 const size_t ga = (size_t)(rD / sry) * nxa + (x0 / srx + c);
                 if (a.heat_s) a.heat_s[ga] = (double)h0 * hscale;
                 if (a.heat_l) a.heat_l[ga] = (double)h1 * hscale;
+                if constexpr (!MANY) break;
             }
             __syncwarp();
             acc_s[0] = acc_s[1] = acc_q[0] = acc_q[1] = splat<V>(0.0f);
@@ -615,7 +619,7 @@ struct WarpStrip4 {
     }
 };
 
-template <bool NC>
+template <bool NC, bool MANY>
 __global__ void __launch_bounds__(kWarp4CtaThreads, 2) k_fire_warp4(const StepArgs a) {
     __shared__ __align__(16) float lut[FIRE_MAX_CLASSES * 8];
     __shared__ __align__(16) float lut2[FIRE_MAX_CLASSES * 12];
@@ -672,7 +676,7 @@ __global__ void __launch_bounds__(kWarp4CtaThreads, 2) k_fire_warp4(const StepAr
     const double tstart = *a.t_in;
     if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0) *a.t_out = tstart + a.dt;
     if (x0 >= a.nx) return;  // whole warp
-    WarpStrip4<NC> s(a, lut, lut2, lutq, hw[w], rows, cols[w]);
+    WarpStrip4<NC, MANY> s(a, lut, lut2, lutq, hw[w], rows, cols[w]);
     s.run(x0, y0, tstart);
     const int stw = __reduce_or_sync(0xffffffffu, s.st);
     if ((threadIdx.x & 31) == 0 && stw) atomicOr(a.status, stw);
@@ -685,10 +689,11 @@ cudaError_t launch_warp4(const StepArgs &a, cudaStream_t s) {
         return cudaErrorInvalidValue;
     const int strips = (a.nx + W - 1) / W;
     dim3 grid((strips + kWarpStrips - 1) / kWarpStrips, (a.ny + L - 1) / L);
+    const bool many = a.kx > 32;
     if (a.nco[0])
-        k_fire_warp4<true><<<grid, kWarp4CtaThreads, 0, s>>>(a);
+        (many ? k_fire_warp4<true, true> : k_fire_warp4<true, false>)<<<grid, kWarp4CtaThreads, 0, s>>>(a);
     else
-        k_fire_warp4<false><<<grid, kWarp4CtaThreads, 0, s>>>(a);
+        (many ? k_fire_warp4<false, true> : k_fire_warp4<false, false>)<<<grid, kWarp4CtaThreads, 0, s>>>(a);
     return cudaGetLastError();
 }
 

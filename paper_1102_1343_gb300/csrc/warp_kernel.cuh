@@ -567,7 +567,7 @@ struct RowStrip {
                     stencil<FORM>(D, Pc, U, l, rr, y0 + k, L, R);
                     WCoef<T> co;
                     coef(e1, co);
-                    const V G = neg_rhs2<T, MODE != ROW_PLAIN>(Pc, L, R, D, U, idx2, idy2, i2dx2, i2dy2,
+                    const V G = neg_rhs2<T, MODE != ROW_PLAIN, true>(Pc, L, R, D, U, idx2, idy2, i2dx2, i2dy2,
                                                                eps2, co, e1.m, un, vn, e1.zx, e1.zy);
                     const unsigned s1 = sl + n1;
                     sts(s1 + S::Q, fma2(ndt2, G, Pc));
@@ -675,7 +675,7 @@ struct RowStrip {
         stencil<FORM>(D, Qc, U, l, rr, r, L, R);
         WCoef<T> co;
         coef(e, co);
-        const V G2 = neg_rhs2<T, MODE != ROW_PLAIN>(Qc, L, R, D, U, idx2, idy2, i2dx2, i2dy2, eps2, co, e.m,
+        const V G2 = neg_rhs2<T, MODE != ROW_PLAIN, true>(Qc, L, R, D, U, idx2, idy2, i2dx2, i2dy2, eps2, co, e.m,
                                                     un, vn, e.zx, e.zy);
         // P0 + dt (F0/2 + F2/2) = P0 - dt/2 (G0 + G2), the halving exact
         const V N0 = fma2(ndth2, add2(lds<V>(s2 + S::FN), G2), P0);
