@@ -143,7 +143,11 @@ __host__ __device__ inline size_t tile_wind_elems(int TX, int TY, int ky) {
 // a warp per row left 18 of 32 lanes idle).  TAB: the wind is interpolated
 // once per node, from rows interpolated in x, with the weights and quotients
 // formed once per column and row of the tile (per node and stage they cost
-// more FP64 than the right-hand side); otherwise per node and stage.  Small
+// more FP64 than the right-hand side); otherwise per node and stage, and the
+// launch is an ordinary one (the code of a chained one alone cost such tiles,
+// which nothing waits for, 10 to 20 %: 1000^2 nodes in FP32, tiles of 80x40, 12
+// steps 0.92 ms with it, 0.88 without; 510^2 in FP64, tiles of 40x40, 4.6 and
+// 4.3, with the linear fuel fraction 8.3 and 6.7).  Small
 // meshes, where this kernel is the default, are bound by the latency of its
 // chain of stages.  Measured, us per step (GB300), before and now: 100^2 nodes
 // in FP64 53.7 and 24.3 (30.0 with the steps not chained, see launch_chained,
@@ -152,7 +156,7 @@ __host__ __device__ inline size_t tile_wind_elems(int TX, int TY, int ky) {
 template <typename T, bool TAB>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 : kTileCtasPerSmF32)
     k_fire_step(const StepArgs a) {
-    chain_go();
+    if (TAB) chain_go();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_status;
     const int tid = threadIdx.x;
@@ -234,7 +238,8 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 :
             P0[e] = val;
         }
     };
-    if (!a.chained) load_psi();
+    const bool chained = TAB && a.chained;
+    if (!chained) load_psi();
     for (int k = tid; k < a.ncls * K_N; k += kThreads) lut[k] = T(a.coef[k]);
     const int jb = max(y0 / sry - 2, 0);  // first wind row of the table
     for (int e = tid; e < WR * BW2; e += kThreads) {
@@ -281,7 +286,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 :
             vn_s[e] = vn;
         }
     }
-    if (a.chained) {
+    if (chained) {
         chain_wait();
         load_psi();
     }
@@ -335,9 +340,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 :
         }
         const size_t g = WF_CHK((size_t)gy * nx + gx, (long long)nx * ny, st);
         const T p0 = P0[(ly + 2) * BW3 + (lx + 2)];
-        // t_i where the node burns already, read ahead of the arithmetic
+        // t_i where the node burns already, read ahead of the arithmetic (in the
+        // small tiles, bound by latency)
         double ti = 0.0;
-        if (full && le0(p0)) ti = a.tign[g];
+        if (TAB && full && le0(p0)) ti = a.tign[g];
         int cls = fuel[g];
         cls = cls > ncm1 ? ncm1 : cls;
         const int c2 = (ly + 1) * BW2 + (lx + 1);
@@ -359,7 +365,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 :
         if (full && le0(pn)) {
             const bool cross = p0 > T(0) && pn <= T(0);
             if (cross || pn < T(0)) {
-                if (!le0(p0)) ti = a.tign[g];
+                if (!TAB || !le0(p0)) ti = a.tign[g];
                 if (cross && isinf(ti)) {
                     const double q0 = (double)p0, q1 = (double)pn;
                     ti = tstart + q0 * a.dt / (q0 - q1);
@@ -709,7 +715,7 @@ cudaError_t launch_step(const StepArgs &a, cudaStream_t s) {
     cudaError_t e = prepare_step_kernel<T>(smem);
     if (e != cudaSuccess) return e;
     return tab ? launch_chained(a.chained, k_fire_step<T, true>, grid, kThreads, tab, s, a)
-               : launch_chained(a.chained, k_fire_step<T, false>, grid, kThreads, smem, s, a);
+               : launch_chained(false, k_fire_step<T, false>, grid, kThreads, smem, s, a);
 }
 
 template <typename T>
