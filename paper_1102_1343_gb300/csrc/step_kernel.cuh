@@ -495,7 +495,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 :
 // order; newly ignited nodes (psi > 0 >= psi_g, no ignition time yet) get
 // the arrival time.
 //
-// A CTA owns a tile of kIgnX x kIgnY nodes.  Its threads read the tile's psi,
+// A CTA owns a tile of 64 x 16 nodes.  Its threads read the tile's psi,
 // and one thread per segment bounds dist - rho over the tile (the distance of
 // the tile's centre to the segment, less or plus the tile's radius).  A
 // segment can change a node of the tile only where it may lie below the
@@ -511,11 +511,28 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? kTileCtasPerSmF64 :
 // kernel took 163 us when every node tested every segment in double, 59 with
 // the exact test's IEEE quotient and root; a step with it takes 69 us (210, 94).
 // ---------------------------------------------------------------------------
-constexpr int kIgnX = 64, kIgnY = 16, kIgnThreads = 256, kIgnPer = kIgnX * kIgnY / kIgnThreads;
+constexpr int kIgnX = 64, kIgnThreads = 256, kIgnRows = kIgnThreads / kIgnX;
 static_assert(kMaxSegPerLaunch <= kIgnThreads, "one thread bounds each segment of a launch");
 
-template <typename T>
+// the exact test of segment s at a node (x, y): its distance less the radius,
+// and the parameter of the segment's nearest point (contracted one way only: the
+// same bits in both forms of the kernel)
+__device__ __forceinline__ double ignition_distance(const IgnSeg &s, double x, double y, double &u, double &d) {
+    const double qx = x - s.ax, qy = y - s.ay;
+    u = fma(qx, s.dx, qy * s.dy) * s.il2;
+    // u limited to [0, 1] on its bits
+    if (__double_as_longlong(u) <= 0) u = 0.0;
+    else if (__double2hiint(u) >= 0x3ff00000) u = 1.0;
+    const double rx = fma(-u, s.dx, qx), ry = fma(-u, s.dy, qy);
+    d = sqrt64(fma(rx, rx, ry * ry));
+    return d - s.rho;
+}
+
+// PER: nodes of a thread, one above the other.  TILES false: every segment is
+// tested at every node.
+template <typename T, int PER, bool TILES>
 __global__ void __launch_bounds__(kIgnThreads) k_ignite(const IgniteArgs a) {
+    constexpr int kIgnY = kIgnRows * PER;
     __shared__ float s_lo[kMaxSegPerLaunch], s_qx[kMaxSegPerLaunch], s_qy[kMaxSegPerLaunch];
     __shared__ int s_list[kMaxSegPerLaunch];
     __shared__ int s_n;
@@ -527,11 +544,11 @@ __global__ void __launch_bounds__(kIgnThreads) k_ignite(const IgniteArgs a) {
     const int x0 = (int)(blockIdx.x % tx) * kIgnX, y0 = (int)(blockIdx.x / tx) * kIgnY;
     const int i = x0 + lx;
     // the tile's psi, and its largest value rounded up
-    T p[kIgnPer];
+    T p[PER];
     float pm = -INFINITY;
 #pragma unroll
-    for (int e = 0; e < kIgnPer; ++e) {
-        const int j = y0 + ly + e * (kIgnThreads / kIgnX);
+    for (int e = 0; e < PER; ++e) {
+        const int j = y0 + ly + e * kIgnRows;
         const bool in = i < a.nx && j < a.ny;
         p[e] = in ? psi[(size_t)j * a.nx + i] : T(0);
         if (in) {
@@ -539,64 +556,67 @@ __global__ void __launch_bounds__(kIgnThreads) k_ignite(const IgniteArgs a) {
             pm = f == f ? fmaxf(pm, f) : INFINITY;
         }
     }
+    int n = a.nseg;
+    if constexpr (TILES) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) pm = fmaxf(pm, __shfl_xor_sync(0xffffffffu, pm, o));
-    if ((tid & 31) == 0) s_pmax[tid >> 5] = pm;
-    // bounds of dist - rho over the tile (float with a margin above its
-    // rounding error: coordinates within 1e-6 of their size)
-    float lo = 0.0f, up = INFINITY;
-    const double xc = ((double)x0 + 0.5 * kIgnX) * a.dx, yc = ((double)y0 + 0.5 * kIgnY) * a.dy;
-    if (tid < a.nseg) {
-        const IgnSeg &s = a.seg[tid];
-        const float qx = (float)(xc - s.ax), qy = (float)(yc - s.ay);
-        const float sx = (float)s.dx, sy = (float)s.dy;
-        const float L2 = sx * sx + sy * sy;
-        float u = L2 > 0.0f ? (qx * sx + qy * sy) / L2 : 0.0f;
-        u = fminf(fmaxf(u, 0.0f), 1.0f);
-        const float rx = qx - u * sx, ry = qy - u * sy;
-        const float d = sqrtf(rx * rx + ry * ry);
-        const float rad = 0.5f * hypotf(kIgnX * (float)a.dx, kIgnY * (float)a.dy);
-        const float eps = 4e-6f * (fabsf(qx) + fabsf(qy) + fabsf(sx) + fabsf(sy) + rad + fabsf((float)s.rho)) + 1e-6f;
-        lo = d - rad - (float)s.rho - eps;
-        up = d + rad - (float)s.rho + eps;
-        s_lo[tid] = lo;
-        s_qx[tid] = qx;
-        s_qy[tid] = qy;
-    }
-    __syncthreads();
-    if (tid < 32) {
-        float m = -INFINITY;
-        for (int k = 0; k < kIgnThreads / 32; ++k) m = fmaxf(m, s_pmax[k]);
-        if (m == -INFINITY) m = INFINITY;  // (no node of the tile is a number below infinity)
-        if (tid == 0) s_up = m;
-    }
-    __syncthreads();
-    if (tid < kMaxSegPerLaunch) {  // warps 0 and 1
-        float m = up;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if ((tid & 31) == 0) s_pmax[tid >> 5] = m;
-    }
-    __syncthreads();
-    if (tid < 32) {
-        const float lim = fminf(s_up, fminf(s_pmax[0], s_pmax[1]));
-        int n = 0;
-        for (int k0 = 0; k0 < a.nseg; k0 += 32) {
-            const int k = k0 + tid;
-            const bool take = k < a.nseg && (!(s_lo[k] > lim) || !(s_lo[k] > 0.0f));
-            const unsigned v = __ballot_sync(0xffffffffu, take);
-            if (take) s_list[n + __popc(v & ((1u << tid) - 1))] = k;
-            n += __popc(v);
+        for (int o = 16; o > 0; o >>= 1) pm = fmaxf(pm, __shfl_xor_sync(0xffffffffu, pm, o));
+        if ((tid & 31) == 0) s_pmax[tid >> 5] = pm;
+        // bounds of dist - rho over the tile (float with a margin above its
+        // rounding error: coordinates within 1e-6 of their size)
+        float lo = 0.0f, up = INFINITY;
+        const double xc = ((double)x0 + 0.5 * kIgnX) * a.dx, yc = ((double)y0 + 0.5 * kIgnY) * a.dy;
+        if (tid < a.nseg) {
+            const IgnSeg &s = a.seg[tid];
+            const float qx = (float)(xc - s.ax), qy = (float)(yc - s.ay);
+            const float sx = (float)s.dx, sy = (float)s.dy;
+            const float L2 = sx * sx + sy * sy;
+            float u = L2 > 0.0f ? (qx * sx + qy * sy) / L2 : 0.0f;
+            u = fminf(fmaxf(u, 0.0f), 1.0f);
+            const float rx = qx - u * sx, ry = qy - u * sy;
+            const float d = sqrtf(rx * rx + ry * ry);
+            const float rad = 0.5f * hypotf(kIgnX * (float)a.dx, kIgnY * (float)a.dy);
+            const float eps = 4e-6f * (fabsf(qx) + fabsf(qy) + fabsf(sx) + fabsf(sy) + rad + fabsf((float)s.rho)) + 1e-6f;
+            lo = d - rad - (float)s.rho - eps;
+            up = d + rad - (float)s.rho + eps;
+            s_lo[tid] = lo;
+            s_qx[tid] = qx;
+            s_qy[tid] = qy;
         }
-        if (tid == 0) s_n = n;
+        __syncthreads();
+        if (tid < 32) {
+            float m = -INFINITY;
+            for (int k = 0; k < kIgnThreads / 32; ++k) m = fmaxf(m, s_pmax[k]);
+            if (m == -INFINITY) m = INFINITY;  // (no node of the tile is a number below infinity)
+            if (tid == 0) s_up = m;
+        }
+        __syncthreads();
+        if (tid < kMaxSegPerLaunch) {  // warps 0 and 1
+            float m = up;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
+            if ((tid & 31) == 0) s_pmax[tid >> 5] = m;
+        }
+        __syncthreads();
+        if (tid < 32) {
+            const float lim = fminf(s_up, fminf(s_pmax[0], s_pmax[1]));
+            int n = 0;
+            for (int k0 = 0; k0 < a.nseg; k0 += 32) {
+                const int k = k0 + tid;
+                const bool take = k < a.nseg && (!(s_lo[k] > lim) || !(s_lo[k] > 0.0f));
+                const unsigned v = __ballot_sync(0xffffffffu, take);
+                if (take) s_list[n + __popc(v & ((1u << tid) - 1))] = k;
+                n += __popc(v);
+            }
+            if (tid == 0) s_n = n;
+        }
+        __syncthreads();
+        n = s_n;
     }
-    __syncthreads();
-    const int n = s_n;
     if (n == 0 || i >= a.nx) return;
     const double x = ((double)i + 0.5) * a.dx;
 #pragma unroll
-    for (int e = 0; e < kIgnPer; ++e) {
-        const int jl = ly + e * (kIgnThreads / kIgnX), j = y0 + jl;
+    for (int e = 0; e < PER; ++e) {
+        const int jl = ly + e * kIgnRows, j = y0 + jl;
         if (j >= a.ny) continue;
         const float ox = ((float)lx + 0.5f - 0.5f * kIgnX) * (float)a.dx, oy = ((float)jl + 0.5f - 0.5f * kIgnY) * (float)a.dy;
         const size_t g = (size_t)j * a.nx + i;
@@ -605,13 +625,13 @@ __global__ void __launch_bounds__(kIgnThreads) k_ignite(const IgniteArgs a) {
         double ti = 0.0;
         bool read = false, changed = false, tchanged = false;
         for (int q = 0; q < n; ++q) {
-            const int k = s_list[q];
+            const int k = TILES ? s_list[q] : q;
             const IgnSeg &s = a.seg[k];
             // skip the segment only when the exact test below can change
             // neither psi (needs dist < psi + rho) nor, psi then being above
             // dist - rho too, the ignition time; delta bounds the error of the
             // distance in float
-            {
+            if constexpr (TILES) {
                 const float qx = s_qx[k] + ox, qy = s_qy[k] + oy;
                 const float sx = (float)s.dx, sy = (float)s.dy;
                 const float L2f = sx * sx + sy * sy;
@@ -624,14 +644,8 @@ __global__ void __launch_bounds__(kIgnThreads) k_ignite(const IgniteArgs a) {
                 const float dl = lim + delta + 1e-6f * fabsf(lim);
                 if (!(dl > 0.0f && !(d2 > dl * dl))) continue;
             }
-            const double qx = x - s.ax, qy = y - s.ay;
-            double u = (qx * s.dx + qy * s.dy) * s.il2;
-            // u limited to [0, 1] on its bits
-            if (__double_as_longlong(u) <= 0) u = 0.0;
-            else if (__double2hiint(u) >= 0x3ff00000) u = 1.0;
-            const double rx = qx - u * s.dx, ry = qy - u * s.dy;
-            const double d = sqrt64(rx * rx + ry * ry);
-            const double pg = d - s.rho;
+            double u, d;
+            const double pg = ignition_distance(s, x, y, u, d);
             if (pe > T(0) && le0(pg)) {
                 if (!read) {
                     ti = a.tign[g];
@@ -641,7 +655,7 @@ __global__ void __launch_bounds__(kIgnThreads) k_ignite(const IgniteArgs a) {
                     if (s.drip) {
                         // the fire starts at the nearest point when the torch
                         // lays it and reaches the node at S_g, by t at the latest
-                        const double ta = (s.tg + u * (s.tlay - s.tg)) + d / s.sg;
+                        const double ta = fma(u, s.tlay - s.tg, s.tg) + d / s.sg;
                         ti = ta < s.tnow ? ta : s.tnow;
                     } else {
                         ti = s.sg > 0.0 ? s.tg + d / s.sg : s.tg;
@@ -720,9 +734,19 @@ cudaError_t launch_step(const StepArgs &a, cudaStream_t s) {
 
 template <typename T>
 cudaError_t launch_ignite(const IgniteArgs &a, cudaStream_t s) {
-    const long long tiles = (long long)((a.nx + kIgnX - 1) / kIgnX) * ((a.ny + kIgnY - 1) / kIgnY);
+    // few nodes, or few tests in all: the bounds of a tile, behind four
+    // barriers, and four nodes to a thread take longer than the tests that
+    // they save.  us per FP32 step with it, every segment at every node and by
+    // tiles: 100^2 nodes, 4 segments 19 and 35, 64 segments 87 and 179; 200^2,
+    // 16 segments 54 and 61, 64 segments 163 and 141; 400^2, 4 segments 46 and
+    // 44, 16 segments 115 and 69; 800^2, 1 segment 54 and 61, 4 segments 112
+    // and 72.
+    const double nodes = (double)a.nx * a.ny;
+    const bool plain = nodes <= 3e4 || nodes * a.nseg <= 7e5;
+    const int rows = kIgnRows * (plain ? 1 : 4);
+    const long long tiles = (long long)((a.nx + kIgnX - 1) / kIgnX) * ((a.ny + rows - 1) / rows);
     if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;  // (beyond 2^41 nodes)
-    k_ignite<T><<<(unsigned)tiles, kIgnThreads, 0, s>>>(a);
+    (plain ? k_ignite<T, 1, false> : k_ignite<T, 4, true>)<<<(unsigned)tiles, kIgnThreads, 0, s>>>(a);
     return cudaGetLastError();
 }
 
