@@ -329,7 +329,7 @@ int configure_kernel(fire_ctx *c, int variant, int kx, int ky) {
         if (W > kWarpMaxColumns || (W & 1) || L > kWarpMaxRows || (long long)c->n > kWarpMaxNodes)
             return FIRE_ERR_ARG;
         if (variant == FIRE_KERNEL_WARP_DENSE && c->prec != FIRE_FP32) return FIRE_ERR_ARG;
-        const int kr = ky < kRowMaxBands ? ky : kRowMaxBands;
+        const int kr = row_strip_bands(c->prec == FIRE_FP64, ky, c->g.sr_y);
         sm = c->prec == FIRE_FP64 ? warp_smem_bytes<double>(kr, c->g.sr_y, c->ncls)
                                   : warp_smem_bytes<float>(kr, c->g.sr_y, c->ncls);
         if (sm > c->smem_max) return FIRE_ERR_ARG;
@@ -604,7 +604,7 @@ int warp_launch_rows(bool fp64, int nx, int ny, int W, int sry, int n_sm) {
     const long strips = cdiv_l(nx, W), slots = (long)n_sm * (fp64 ? kRowCtasPerSmF64 : kRowCtasPerSmF32);
     int best = 1;
     double least = 0;
-    for (int ky = 1; ky <= kRowMaxBands && (ky == 1 || (ky - 1) * (long)sry < ny) && (ky == 1 || ky * (long)sry <= kWarpMaxRows); ++ky) {
+    for (int ky = 1; ky <= row_max_bands(fp64, sry) && (ky == 1 || (ky - 1) * (long)sry < ny) && (ky == 1 || ky * (long)sry <= kWarpMaxRows); ++ky) {
         const long L = (long)ky * sry;
         const double t = (double)(strips * cdiv_l(ny, L)) * (L + 10) / slots + 0.8 * (L + 20);
         if (ky == 1 || t < least) {

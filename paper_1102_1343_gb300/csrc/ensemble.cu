@@ -298,7 +298,7 @@ int ens_plan(fire_ensemble *e) {
         double t;
         ctx_info(e->members[m], &prec, &variant, &nx, &ny, &srx, &sry, &kx, &ky, &ncls, &cur, &t);
         if (variant != e->variant) return FIRE_ERR_STATE;
-        if (e->variant == FIRE_KERNEL_WARP) ky = row_strip_bands(ky, sry);
+        if (e->variant == FIRE_KERNEL_WARP) ky = row_strip_bands(e->prec == FIRE_FP64, ky, sry);
         const int W = kx * srx, L = ky * sry;
         const int count = ((nx + W - 1) / W) * ((ny + L - 1) / L);
         for (int y0 = 0; y0 < ny; y0 += L)
@@ -552,7 +552,7 @@ int fire_ensemble_step(fire_ensemble *e, int nsteps, double dt, const void *cons
                                           e->margs_host[2 * m + p]);
                     if (r) return r;
                     StepArgs &ma = e->margs_host[2 * m + p];
-                    if (e->variant == FIRE_KERNEL_WARP) ma.ky = row_strip_bands(ma.ky, ma.sry);
+                    if (e->variant == FIRE_KERNEL_WARP) ma.ky = row_strip_bands(e->prec == FIRE_FP64, ma.ky, ma.sry);
                 }
             }
             e->run_host->t0 = t0;

@@ -178,7 +178,14 @@ constexpr int kRowCtasPerSmF32 = 6;  // its resident CTAs per SM that the regist
 constexpr int kRowCtasPerSmF64 = 2;
 constexpr int kTileCtasPerSmF32 = 4;  // and of the tile kernel
 constexpr int kTileCtasPerSmF64 = 2;
-constexpr int kRowMaxBands = 16;     // atmospheric rows of one CTA of it at most
+// atmospheric rows of one CTA of it at most (the wind table of a CTA: at
+// refinement 1, where 16 are few, 28 keep the five CTAs per SM of 16 in FP32;
+// 8000^2 nodes there, six steps 11.2 ms with 16, 9.8 with 28)
+constexpr int row_max_bands(bool fp64, int sry) { return !fp64 && sry == 1 ? 28 : 16; }
+// a taller strip is cut into CTAs of that many (the results do not depend on it)
+constexpr int row_strip_bands(bool fp64, int ky, int sry) {
+    return ky < row_max_bands(fp64, sry) ? ky : row_max_bands(fp64, sry);
+}
 constexpr int kWarpStrips = 4;       // warps (strips) per CTA of the four-column warp kernel
 constexpr int kWarpMaxColumns = 60;  // output columns of one warp strip (even)
 constexpr int kWarpMaxRows = 512;    // output rows of one warp strip

@@ -895,10 +895,6 @@ struct RowStrip {
     }
 };
 
-// a strip taller than kRowMaxBands atmospheric rows is cut into CTAs of at
-// most that many (the wind table of a CTA); the results do not depend on it
-inline int row_strip_bands(int ky, int sry) { return ky < kRowMaxBands ? ky : kRowMaxBands; }
-
 template <typename T, int MODE, int WIDTH, bool FULL>
 __global__ void __launch_bounds__(32 * kRowWarps, (row_ctas<T, MODE>())) k_fire_warp(const StepArgs a) {
     extern __shared__ __align__(16) unsigned char row_smem[];
@@ -962,7 +958,7 @@ cudaError_t launch_warp(const StepArgs &args, cudaStream_t s) {
     if (W > kWarpMaxColumns || (W & 1) || W < 2 || a.ky * a.sry > kWarpMaxRows ||
         (long long)a.nx * a.ny > kWarpMaxNodes)
         return cudaErrorInvalidValue;
-    a.ky = row_strip_bands(a.ky, a.sry);
+    a.ky = row_strip_bands(sizeof(T) == 8, a.ky, a.sry);
     const int L = a.ky * a.sry;
     const unsigned bands = (a.ny + L - 1) / L, rows = bands < 65535u ? bands : 65535u;
     const dim3 grid((a.nx + W - 1) / W, rows, (bands + rows - 1) / rows);
