@@ -363,7 +363,7 @@ def run_gpu(args, rank, world):
         pkg.fire_set_kernel(m.ctx, *args.kernel)
     elif args.autotune:
         m.autotune(u, v, w.dt, probe_steps=3)  # the library's own tuner, before timing
-    kernel = pkg.fire_get_kernel(m.ctx)
+    kernel = pkg.fire_get_launch(m.ctx)
     stream = torch.cuda.current_stream(dev)
 
     for _ in range(args.warmup):
@@ -386,7 +386,7 @@ def run_gpu(args, rank, world):
     # the adaptive kernel choice counts burnt nodes every 64 steps (one small
     # kernel each, inside the timed region)
     _, counts1, burnt_seen = pkg.fire_adaptive_info(m.ctx)
-    kernel_end = pkg.fire_get_kernel(m.ctx)
+    kernel_end = pkg.fire_get_launch(m.ctx)
     clk = clocks.stop() if rank == 0 else {}
     ms = max_over_ranks(e0.elapsed_time(e1), dev, world)
     value = whole_job_rate(cells, args.steps, world, ms / 1000.0)
@@ -579,7 +579,7 @@ def bench_burning(pkg, dev, steps):
         k_ms, k_n = pkg.fire_kernel_time_ms(m.ctx)
         pkg.fire_enable_timing(m.ctx, False)
         k_avg = k_ms / max(1, k_n)
-        kernel = pkg.fire_get_kernel(m.ctx)
+        kernel = pkg.fire_get_launch(m.ctx)
         achieved = BYTES_PER_CELL_STEP["fp32"] * cells / (k_avg / 1000.0) / 1e9
         return {"value": cells * steps / (ms / 1e3), "unit": UNIT, "steps": steps,
                 "ms_per_step": ms / steps, "kernel_ms": k_avg,

@@ -325,10 +325,8 @@ double fire_time(const fire_ctx *ctx);
  *                      columns (an even number <= 60) and ky*sr_y rows, each
  *                      warp with one row of every stage at a time, neighbours
  *                      exchanged by shuffles and through rings of rows in
- *                      shared memory; strips of more than 16 atmospheric rows
- *                      are cut, and fire_init's default strips run with the
- *                      rows per CTA that suit the mesh and the device (no
- *                      result depends on either);
+ *                      shared memory (cut into CTAs of fewer rows, see
+ *                      fire_get_launch; no result depends on it);
  *   FIRE_KERNEL_WARP4  (FIRE_FP32 only) each warp marches alone down a strip
  *                      of kx*sr_x <= 120 columns, four columns per lane, rows
  *                      held in registers;
@@ -386,7 +384,21 @@ int fire_adaptive_info(const fire_ctx *ctx, int *on, long long *counts, double *
  * scheme. */
 enum fire_fraction_scheme { FIRE_FRACTION_SUBCELL = 0, FIRE_FRACTION_LINEAR = 1 };
 int fire_set_fraction_scheme(fire_ctx *ctx, int scheme);
+
+/* The kernel the context is configured with: the default of its mesh
+ * (fire_default_kernel; under the adaptive choice the shape of its current
+ * name), or the last one set.  Outputs nullable. */
 int fire_get_kernel(const fire_ctx *ctx, int *variant, int *kx, int *ky);
+
+/* The kernel and shape per CTA that the context's launches take.  A shape set by
+ * fire_set_kernel is launched as it stands (FIRE_KERNEL_WARP_DENSE as
+ * FIRE_KERNEL_WARP, strips of more than 16 atmospheric rows, 28 at refinement 1
+ * in FIRE_FP32, cut into CTAs of as many).  fire_init's default stands for the
+ * form that is fastest for the mesh and the device, with the same results bit
+ * for bit: warp strips with other rows per CTA, FIRE_FP64 marching strips as warp
+ * strips, one-cell tiles merged.  Setting the shape that fire_get_kernel reports
+ * therefore fixes it, and can be slower.  Outputs nullable. */
+int fire_get_launch(const fire_ctx *ctx, int *variant, int *kx, int *ky);
 
 /* Autotuner of the step kernel: times candidate shapes (the marching strip
  * with widths of about 16..248 columns and heights of about 8..512 rows; the
@@ -398,9 +410,10 @@ int fire_get_kernel(const fire_ctx *ctx, int *variant, int *kx, int *ky);
 int fire_autotune(fire_ctx *ctx, const void *wind_u_dev, const void *wind_v_dev, double dt,
                   int probe_steps, int *variant, int *kx, int *ky);
 
-/* The launch shape fire_init (and fire_step_noalloc) takes by default for a
- * mesh of nx_atm x ny_atm atmospheric cells refined sr_x x sr_y, in the given
- * precision, on a device with n_sm SMs: strips (warp strips in FP32 when
+/* The kernel and shape that fire_init configures by default (and
+ * fire_step_noalloc takes as its own default; fire_get_launch tells what a
+ * context launches for it) for a mesh of nx_atm x ny_atm atmospheric cells
+ * refined sr_x x sr_y, in the given precision, on a device with n_sm SMs: strips (warp strips in FP32 when
  * sr_x <= 30, else marching strips) as tall as the large-mesh shapes (~160 /
  * ~60 rows) while that still gives 3.5 / 2.5 waves of resident CTAs, else
  * shorter, down to one atmospheric cell; 2-D tiles of one atmospheric cell

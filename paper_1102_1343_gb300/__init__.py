@@ -58,7 +58,7 @@ ABI_SYMBOLS = ("fire_init", "fire_step", "fire_step_host", "fire_run", "fire_get
                "fire_default_kernel", "fire_adjoint_heat", "fire_set_moisture",
                "fire_wind_at_height", "fire_heat_insertion", "fire_set_fraction_scheme",
                "fire_bounds_checked", "fire_bounds_selftest", "fire_set_adaptive",
-               "fire_adaptive_info")
+               "fire_adaptive_info", "fire_get_launch")
 FIRE_FRACTION_SUBCELL = 0
 FIRE_FRACTION_LINEAR = 1
 
@@ -133,6 +133,7 @@ def load_library(path: str | None = None):
     L.fire_adaptive_info.argtypes = [_P, C.POINTER(C.c_int), C.POINTER(C.c_longlong),
                                      C.POINTER(C.c_double)]
     L.fire_get_kernel.argtypes = [_P, C.POINTER(C.c_int), C.POINTER(C.c_int), C.POINTER(C.c_int)]
+    L.fire_get_launch.argtypes = [_P, C.POINTER(C.c_int), C.POINTER(C.c_int), C.POINTER(C.c_int)]
     L.fire_enable_timing.argtypes = [_P, C.c_int]
     L.fire_kernel_time_ms.argtypes = [_P, C.POINTER(C.c_double), C.POINTER(C.c_long)]
     L.fire_strerror.argtypes = [C.c_int]
@@ -360,8 +361,9 @@ def fire_set_kernel(ctx, variant, kx, ky) -> int:
 
 
 def fire_default_kernel(precision, nx_atm, ny_atm, sr_x, sr_y, n_sm):
-    """(variant, kx, ky) that fire_init takes by default on a device with
-    n_sm SMs (host computation, no device needed)."""
+    """(variant, kx, ky) that fire_init configures by default on a device with
+    n_sm SMs (host computation, no device needed; fire_get_launch tells what a
+    context launches for it)."""
     v, kx, ky = C.c_int(), C.c_int(), C.c_int()
     prec = {"fp32": FIRE_FP32, "fp64": FIRE_FP64}.get(precision, precision)
     _check(load_library().fire_default_kernel(int(prec), int(nx_atm), int(ny_atm), int(sr_x),
@@ -386,6 +388,14 @@ def fire_get_kernel(ctx):
     v, kx, ky = C.c_int(), C.c_int(), C.c_int()
     _check(load_library().fire_get_kernel(ctx, C.byref(v), C.byref(kx), C.byref(ky)),
            "fire_get_kernel")
+    return v.value, kx.value, ky.value
+
+
+def fire_get_launch(ctx):
+    """(variant, kx, ky) that the context's launches take: the shape set, or the
+    form that stands for fire_init's default on this mesh and device."""
+    v, kx, ky = C.c_int(), C.c_int(), C.c_int()
+    _check(load_library().fire_get_launch(ctx, C.byref(v), C.byref(kx), C.byref(ky)), "fire_get_launch")
     return v.value, kx.value, ky.value
 
 

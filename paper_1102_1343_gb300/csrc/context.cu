@@ -1386,6 +1386,15 @@ int fire_get_kernel(const fire_ctx *c, int *variant, int *kx, int *ky) {
     return FIRE_OK;
 }
 
+int fire_get_launch(const fire_ctx *c, int *variant, int *kx, int *ky) {
+    if (!c) return FIRE_ERR_ARG;
+    const bool rows = c->launch.variant == FIRE_KERNEL_WARP || c->launch.variant == FIRE_KERNEL_WARP_DENSE;
+    if (variant) *variant = rows ? FIRE_KERNEL_WARP : c->launch.variant;
+    if (kx) *kx = c->launch.kx;
+    if (ky) *ky = rows ? row_strip_bands(c->prec == FIRE_FP64, c->launch.ky, c->g.sr_y) : c->launch.ky;
+    return FIRE_OK;
+}
+
 int fire_enable_timing(fire_ctx *c, int on) {
     if (!c) return FIRE_ERR_ARG;
     DeviceGuard dg(c->device);

@@ -1,0 +1,46 @@
+"""fire_get_launch tells the kernel and shape that a context's launches take:
+fire_init's default in the form that stands for it, a shape set explicitly as it
+stands, the same before and after the adaptive choice changes its name."""
+import ctypes as C
+
+import pytest
+
+from paper_1102_1343_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    from paper_1102_1343_gb300 import build
+    build.build()
+    import paper_1102_1343_gb300 as p
+    p.load_library()
+    return p
+
+
+def model(pkg, nxa, nya, sr, prec, radius=10.0, steps=1):
+    w = synth.random_landscape(nxa, nya, sr=sr, dx_atm=6.0 * sr, seed=3, ignition="center", ignition_radius=radius, steps=steps)
+    if radius != 10.0:
+        w.ignitions = [synth.point_ignition(w.nx * w.dx / 2, w.ny * w.dy / 2, radius=radius)]
+    return w, pkg.FireModel.from_workload(w, precision=prec)
+
+
+def test_forms_of_the_default(pkg):
+    T, M, W = pkg.FIRE_KERNEL_TILE, pkg.FIRE_KERNEL_MARCH, pkg.FIRE_KERNEL_WARP
+    for nxa, nya, sr, prec, kind, launched in ((51, 51, 10, "fp64", M, W), (200, 150, 10, "fp32", W, W),
+                                               (40, 30, 10, "fp32", T, T), (20, 20, 40, "fp64", M, M)):
+        _, m = model(pkg, nxa, nya, sr, prec)
+        shape, launch = pkg.fire_get_kernel(m.ctx), pkg.fire_get_launch(m.ctx)
+        assert shape[0] == kind and launch[0] == launched
+        if (kind, launched) == (T, T):
+            assert shape == (T, 1, 1) and launch[1] * launch[2] > 1
+        m.close()
+    for var, k, want in ((W, (6, 40), (W, 6, 16)), (pkg.FIRE_KERNEL_WARP_DENSE, (6, 3), (W, 6, 3)), (T, (2, 3), (T, 2, 3)),
+                         (pkg.FIRE_KERNEL_WARP4, (12, 40), (pkg.FIRE_KERNEL_WARP4, 12, 40))):
+        _, m = model(pkg, 51, 51, 10, "fp32")
+        pkg.fire_set_kernel(m.ctx, var, *k)
+        assert pkg.fire_get_kernel(m.ctx) == (var, *k) and pkg.fire_get_launch(m.ctx) == want
+        m.close()
+    i = C.c_int()
+    assert pkg.load_library().fire_get_launch(None, C.byref(i), C.byref(i), C.byref(i)) == pkg.FIRE_ERR_ARG
