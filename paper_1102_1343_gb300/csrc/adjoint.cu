@@ -1535,7 +1535,6 @@ int run_adjoint(fire_ctx *c, int nsteps, double dt, const void *u, const void *v
     auto launch_step_kernel = [&](const StepArgs &ra, cudaStream_t cs) -> cudaError_t {
         return variant == FIRE_KERNEL_MARCH   ? launch_march<T>(ra, cs)
                : variant == FIRE_KERNEL_WARP  ? launch_warp<T>(ra, cs)
-               : variant == FIRE_KERNEL_WARP_DENSE ? launch_warp<T>(ra, cs)
                : variant == FIRE_KERNEL_WARP4 ? (sizeof(T) == 4 ? launch_warp4(ra, cs)
                                                                 : cudaErrorInvalidValue)
                                               : launch_step<T>(ra, cs);
@@ -1782,8 +1781,7 @@ int run_adjoint(fire_ctx *c, int nsteps, double dt, const void *u, const void *v
     // the reverse steps need psi alone of the recomputed states: the kernels
     // that can leave out the rest do (the adjoint of 100 steps of 510^2 nodes
     // with moisture, FP32: 6.85 -> 6.04 ms; of 60 of 370x290: 4.33 -> 4.08)
-    const bool psi_alone = variant == FIRE_KERNEL_WARP || variant == FIRE_KERNEL_WARP_DENSE ||
-                           variant == FIRE_KERNEL_TILE;
+    const bool psi_alone = variant == FIRE_KERNEL_WARP || variant == FIRE_KERNEL_TILE;
 
     // One segment: ring slot 0 holds its checkpoint and tseg its step times,
     // so every segment of a given length issues the same launches: the

@@ -50,7 +50,8 @@ struct fire_ctx {
 
     int variant = FIRE_KERNEL_MARCH;
     int kx = 0, ky = 0;
-    DefaultShape launch{FIRE_KERNEL_MARCH, 0, 0};  // kernel and shape of its launches (launch_shape)
+    DefaultShape launch{FIRE_KERNEL_MARCH, 0, 0};  // kernel and shape of its launches
+    bool by_rule = false;  // launch_shape chose them (fire_init's default, under either name)
     int scheme = 0;  // fuel fraction: 0 subcell scheme, 1 exact for linear data (tiles)
     size_t smem = 0;
     size_t smem_max = 0;
@@ -86,7 +87,6 @@ struct fire_ctx {
     bool adaptive = false;
     bool ad_dense = false;                       // the dense variant is chosen
     int ad_kx = 0, ad_ky = 0, ad_dense_ky = 0;   // the two shapes
-    bool ad_launch = false;                      // launches by launch_shape (fire_init's default)
     unsigned long long *ad_count_dev = nullptr;  // nodes with psi <= 0
     unsigned long long *ad_count_host = nullptr; // page-locked copy of it
     cudaEvent_t ad_ready = nullptr;              // that copy has landed
@@ -235,8 +235,6 @@ cudaError_t launch_variant(const fire_ctx *c, const StepArgs &a, cudaStream_t s)
         return c->prec == FIRE_FP64 ? launch_warp<double>(a, s) : launch_warp<float>(a, s);
     if (c->launch.variant == FIRE_KERNEL_WARP4)
         return c->prec == FIRE_FP32 ? launch_warp4(a, s) : cudaErrorInvalidValue;
-    if (c->launch.variant == FIRE_KERNEL_WARP_DENSE)
-        return c->prec == FIRE_FP32 ? launch_warp<float>(a, s) : cudaErrorInvalidValue;
     return c->prec == FIRE_FP64 ? launch_step<double>(a, s) : launch_step<float>(a, s);
 }
 
@@ -353,15 +351,18 @@ int configure_kernel(fire_ctx *c, int variant, int kx, int ky) {
     c->variant = variant;
     c->kx = kx;
     c->ky = ky;
-    c->launch = DefaultShape{variant, kx, ky};
+    // (both names of the row kernel launch the same one)
+    c->launch = DefaultShape{variant == FIRE_KERNEL_WARP_DENSE ? FIRE_KERNEL_WARP : variant, kx, ky};
+    c->by_rule = false;
     c->smem = sm;
     return FIRE_OK;
 }
 
 // what launches take in place of the default shape
 void default_launch(fire_ctx *c) {
-    c->launch = launch_shape(c->prec == FIRE_FP64, DefaultShape{c->variant, c->kx, c->ky}, c->g.nx_atm,
+    c->launch = launch_shape(c->prec == FIRE_FP64, DefaultShape{c->launch.variant, c->kx, c->ky}, c->g.nx_atm,
                              c->g.ny_atm, c->g.sr_x, c->g.sr_y, c->ncls, c->n_sm, c->smem_max);
+    c->by_rule = true;
 }
 
 // marching strips of up to 248 columns (an even number) x ~60 rows
@@ -416,7 +417,8 @@ int default_kernel(fire_ctx *c) {
 
 // burnt fraction at which the dense variant takes over, and below which the
 // default strips come back (both names are the row kernel now, launched with
-// the rows of warp_launch_rows: the choice changes no time of a default context)
+// the rows of warp_launch_rows: for a default context the choice changes neither
+// the launches nor the captured graph)
 constexpr double kAdaptOn = 0.005, kAdaptOff = 0.0025;
 constexpr long kAdaptEvery = 64;  // steps between counts
 
@@ -441,11 +443,12 @@ int adaptive_decide(fire_ctx *c, unsigned long long count) {
     c->ad_fraction = (double)count / (double)c->n;
     const bool dense = c->ad_dense ? c->ad_fraction >= kAdaptOff : c->ad_fraction >= kAdaptOn;
     if (dense == c->ad_dense) return FIRE_OK;
+    const bool by_rule = c->by_rule;
     const int r = configure_kernel(c, dense ? FIRE_KERNEL_WARP_DENSE : FIRE_KERNEL_WARP, c->ad_kx,
                                    dense ? c->ad_dense_ky : c->ad_ky);
     if (r != FIRE_OK) return r;
     c->ad_dense = dense;
-    if (c->ad_launch) default_launch(c);
+    if (by_rule) default_launch(c);
     return FIRE_OK;
 }
 
@@ -503,7 +506,6 @@ void adaptive_setup(fire_ctx *c) {
     c->ad_dense = false;
     c->ad_kx = c->kx;
     c->ad_ky = c->ky;
-    c->ad_launch = c->launch != DefaultShape{c->variant, c->kx, c->ky};
     const int short_rows = 60 / c->g.sr_y;
     c->ad_dense_ky = c->ky < short_rows ? c->ky : (short_rows < 1 ? 1 : short_rows);
     c->ad_steps = kAdaptEvery;  // count before the first step
@@ -619,7 +621,7 @@ DefaultShape launch_shape(bool fp64, const DefaultShape &d, int nx_atm, int ny_a
                           int ncls, int n_sm, size_t smem_max) {
     const long long nx = (long long)nx_atm * srx, ny = (long long)ny_atm * sry;
     DefaultShape r = d;
-    if (d.variant == FIRE_KERNEL_WARP || d.variant == FIRE_KERNEL_WARP_DENSE) {
+    if (d.variant == FIRE_KERNEL_WARP) {
         r.ky = warp_launch_rows(fp64, (int)nx, (int)ny, d.kx * srx, sry, n_sm);
     } else if (d.variant == FIRE_KERNEL_MARCH && fp64) {
         int kx = kWarpMaxColumns / srx;
@@ -1199,10 +1201,11 @@ int fire_set_adaptive(fire_ctx *c, int on) {
         return FIRE_ERR_ARG;
     // the current strips become the default shape; the dense variant takes
     // the rows of the shorter strips
-    const bool dense = c->variant == FIRE_KERNEL_WARP_DENSE;
+    const bool dense = c->variant == FIRE_KERNEL_WARP_DENSE, by_rule = c->by_rule;
     if (dense) {
         const int r = configure_kernel(c, FIRE_KERNEL_WARP, c->kx, c->ky);
         if (r) return r;
+        if (by_rule) default_launch(c);
     }
     adaptive_setup(c);
     return FIRE_OK;
@@ -1388,8 +1391,8 @@ int fire_get_kernel(const fire_ctx *c, int *variant, int *kx, int *ky) {
 
 int fire_get_launch(const fire_ctx *c, int *variant, int *kx, int *ky) {
     if (!c) return FIRE_ERR_ARG;
-    const bool rows = c->launch.variant == FIRE_KERNEL_WARP || c->launch.variant == FIRE_KERNEL_WARP_DENSE;
-    if (variant) *variant = rows ? FIRE_KERNEL_WARP : c->launch.variant;
+    const bool rows = c->launch.variant == FIRE_KERNEL_WARP;
+    if (variant) *variant = c->launch.variant;
     if (kx) *kx = c->launch.kx;
     if (ky) *ky = rows ? row_strip_bands(c->prec == FIRE_FP64, c->launch.ky, c->g.sr_y) : c->launch.ky;
     return FIRE_OK;

@@ -44,3 +44,28 @@ def test_forms_of_the_default(pkg):
         m.close()
     i = C.c_int()
     assert pkg.load_library().fire_get_launch(None, C.byref(i), C.byref(i), C.byref(i)) == pkg.FIRE_ERR_ARG
+
+
+@pytest.mark.parametrize("nxa,nya,sr", [(200, 200, 10), (300, 140, 7), (560, 560, 10)])
+def test_adaptive_choice_keeps_the_launches(pkg, nxa, nya, sr):
+    """Sparse, then burning, then sparse again, and the choice turned on anew: the
+    name changes, the launches of a default context do not (on 560 x 560 cells
+    the default rows and the launch's are the same)."""
+    w, m = model(pkg, nxa, nya, sr, "fp32")
+    torch = m.torch
+    shape, launch = pkg.fire_get_kernel(m.ctx), pkg.fire_get_launch(m.ctx)
+    assert shape[0] == pkg.FIRE_KERNEL_WARP
+    u, v = m.wind(w.u, w.v)
+    psi, tign, frac, t = m.state()
+    for burnt in (True, False, True):
+        p = torch.where(torch.arange(m.ny, device="cuda")[:, None] < m.ny // 3, -psi.abs(), psi.abs()) if burnt else psi
+        m.set_state(p, torch.where(p <= 0, -9.0, torch.inf).double(), frac, t)
+        m.step(u, v, 0.25)
+        torch.cuda.synchronize()
+        m.step(u, v, 0.25)  # the count has landed
+        name = pkg.fire_get_kernel(m.ctx)[0]
+        assert name == (pkg.FIRE_KERNEL_WARP_DENSE if burnt else pkg.FIRE_KERNEL_WARP)
+        assert pkg.fire_get_launch(m.ctx) == launch
+    pkg.fire_set_adaptive(m.ctx, True)
+    assert pkg.fire_get_kernel(m.ctx)[0] == pkg.FIRE_KERNEL_WARP and pkg.fire_get_launch(m.ctx) == launch
+    m.close()
