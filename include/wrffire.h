@@ -400,11 +400,12 @@ int fire_get_kernel(const fire_ctx *ctx, int *variant, int *kx, int *ky);
  * therefore fixes it, and can be slower.  Outputs nullable. */
 int fire_get_launch(const fire_ctx *ctx, int *variant, int *kx, int *ky);
 
-/* Autotuner of the step kernel: times candidate shapes (the marching strip
+/* Autotuner of the step kernel: times candidate shapes (the kernel that the
+ * context has and fire_init's default, each as it is launched; the marching strip
  * with widths of about 16..248 columns and heights of about 8..512 rows; the
  * 2-D tile at a few shapes) for probe_steps launches each on a scratch copy
- * of the current state with the given wind and dt, keeps the fastest
- * (fire_set_kernel) and reports it (outputs nullable).  The state and the
+ * of the current state with the given wind and dt, keeps the fastest and
+ * reports it (outputs nullable; as fire_get_kernel and fire_get_launch do).  The state and the
  * model time are unchanged; the scratch is the context's workspace.
  * Synchronous. */
 int fire_autotune(fire_ctx *ctx, const void *wind_u_dev, const void *wind_v_dev, double dt,

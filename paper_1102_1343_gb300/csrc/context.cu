@@ -1244,8 +1244,8 @@ int fire_set_fraction_scheme(fire_ctx *c, int scheme) {
     return FIRE_OK;
 }
 
-// Candidate step-kernel shapes timed on a scratch copy of the state: the
-// marching strip over widths of about 16..248 columns and heights of about
+// Candidate step-kernel shapes timed on a scratch copy of the state: the kernel
+// that the context has, the mesh's default as it is launched, the marching strip over widths of about 16..248 columns and heights of about
 // 8..512 rows, and the 2-D tile over a few shapes; the fastest average of
 // probe_steps launches (after one warm-up launch) is kept.
 int fire_default_kernel(int precision, int nx_atm, int ny_atm, int sr_x, int sr_y, int n_sm,
@@ -1284,6 +1284,7 @@ int fire_autotune(fire_ctx *c, const void *u, const void *v, double dt, int prob
 
     struct Cand {
         int variant, kx, ky;
+        bool by_rule;  // launched in the form that stands for the default
     };
     std::vector<Cand> cands;
     const int srx = c->g.sr_x, sry = c->g.sr_y, nxa = c->g.nx_atm, nya = c->g.ny_atm;
@@ -1297,8 +1298,18 @@ int fire_autotune(fire_ctx *c, const void *u, const void *v, double dt, int prob
             else return;
         }
         for (const Cand &q : cands)
-            if (q.variant == variant && q.kx == kx && q.ky == ky) return;
-        cands.push_back(Cand{variant, kx, ky});
+            if (!q.by_rule && q.variant == variant && q.kx == kx && q.ky == ky) return;
+        cands.push_back(Cand{variant, kx, ky, false});
+    };
+    // the kernel that the context has, and the mesh's default
+    cands.push_back(Cand{c->variant, c->kx, c->ky, c->by_rule});
+    const DefaultShape d = default_shape(c->prec == FIRE_FP64, nxa, nya, srx, sry, c->n_sm);
+    if (!c->by_rule && (c->scheme == 0 || d.variant == FIRE_KERNEL_TILE))
+        cands.push_back(Cand{d.variant, d.kx, d.ky, true});
+    auto take = [&](const Cand &q) {
+        const int rc = configure_kernel(c, q.variant, q.kx, q.ky);
+        if (rc == FIRE_OK && q.by_rule) default_launch(c);
+        return rc;
     };
     if (srx <= kMarchMaxColumns / 2) {
         const int widths[] = {16, 24, 32, 48, 64, 96, 128, 176, 248};
@@ -1330,15 +1341,14 @@ int fire_autotune(fire_ctx *c, const void *u, const void *v, double dt, int prob
         for (int W : widths)
             for (int L : heights) add(FIRE_KERNEL_TILE, W / srx, L / sry);
     }
-    const int save_variant = c->variant, save_kx = c->kx, save_ky = c->ky;
     cudaEvent_t e0, e1;
     WF_CHECK(cudaEventCreate(&e0));
     WF_CHECK(cudaEventCreate(&e1));
     float best = 0.f;
-    Cand win{save_variant, save_kx, save_ky};
+    Cand win = cands[0];
     bool found = false;
     for (const Cand &q : cands) {
-        if (configure_kernel(c, q.variant, q.kx, q.ky) != FIRE_OK) continue;
+        if (take(q) != FIRE_OK) continue;
         // the same starting state for every candidate
         WF_CHECK(cudaMemcpyAsync(sp[0], c->psi[c->cur], N * E, cudaMemcpyDeviceToDevice, c->stream));
         WF_CHECK(cudaMemcpyAsync(sf[0], c->frac[c->cur], N * E, cudaMemcpyDeviceToDevice, c->stream));
@@ -1358,6 +1368,7 @@ int fire_autotune(fire_ctx *c, const void *u, const void *v, double dt, int prob
             a.F_out = sf[(k + 1) & 1];
             a.t_in = stm + (k & 1);
             a.t_out = stm + ((k + 1) & 1);
+            a.chained = k > 1;  // (tiles, as fire_run launches them)
             WF_CHECK(launch_variant(c, a, c->stream));
         }
         WF_CHECK(cudaEventRecord(e1, c->stream));
@@ -1372,7 +1383,7 @@ int fire_autotune(fire_ctx *c, const void *u, const void *v, double dt, int prob
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    r = configure_kernel(c, win.variant, win.kx, win.ky);
+    r = take(win);
     if (r) return r;
     c->adaptive = false;  // the measured choice stays
     if (variant_out) *variant_out = win.variant;

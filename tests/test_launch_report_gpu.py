@@ -69,3 +69,28 @@ def test_adaptive_choice_keeps_the_launches(pkg, nxa, nya, sr):
     pkg.fire_set_adaptive(m.ctx, True)
     assert pkg.fire_get_kernel(m.ctx)[0] == pkg.FIRE_KERNEL_WARP and pkg.fire_get_launch(m.ctx) == launch
     m.close()
+
+
+@pytest.mark.parametrize("n,prec", [(10, "fp64"), (51, "fp64"), (40, "fp32")])
+def test_autotune_leaves_no_context_slower(pkg, n, prec):
+    """The form that stands for the default is among the candidates: after
+    fire_autotune 200 steps take at most 1.2 times as long as before."""
+    import torch
+    w, m = model(pkg, n, n, 10, prec)
+    u, v = m.wind(w.u, w.v)
+    e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+
+    def ms():
+        best = 1e9
+        for _ in range(4):
+            e[0].record()
+            m.run(200, u, v, 0.01)
+            e[1].record()
+            torch.cuda.synchronize()
+            best = min(best, e[0].elapsed_time(e[1]))
+        return best
+
+    before = ms()
+    assert m.autotune(u, v, 0.01) == pkg.fire_get_kernel(m.ctx)
+    assert ms() <= 1.2 * before
+    m.close()
