@@ -266,14 +266,16 @@ def make_classes(classes) -> C.Array:
     arr = (fire_fuel_class * len(classes))()
     for k, c in enumerate(classes):
         # one record per class (a setattr per field took most of the host time
-        # of fire_step_noalloc: 13 classes 25 us, now 9); a field left out, or
-        # a value that only float() or int() takes, goes field by field
-        try:
-            w, b, tf, ch, *rest = _class_values(c)
-            _CLASS_RECORD.pack_into(arr, k * _CLASS_RECORD.size, w, b, int(tf), int(ch), *rest)
-            continue
-        except (KeyError, TypeError, ValueError, OverflowError, struct.error):
-            pass
+        # of fire_step_noalloc: 13 classes 25 us, now 9); a field left out, a
+        # value that only float() or int() takes, or another mapping (which may
+        # make up what it does not hold) goes field by field
+        if type(c) is dict:
+            try:
+                w, b, tf, ch, *rest = _class_values(c)
+                _CLASS_RECORD.pack_into(arr, k * _CLASS_RECORD.size, w, b, int(tf), int(ch), *rest)
+                continue
+            except (KeyError, TypeError, ValueError, OverflowError, struct.error):
+                pass
         for name, typ in fire_fuel_class._fields_:
             val = c.get(name, 0)
             setattr(arr[k], name, int(val) if typ is C.c_int else float(val))
