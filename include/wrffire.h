@@ -352,8 +352,10 @@ int fire_set_kernel(fire_ctx *ctx, int variant, int kx, int ky);
  * the nodes with psi <= 0 on the context's stream; the count is read on a
  * later step without waiting (a host that runs ahead of the device sees it,
  * and changes the kernel, that much later).  From a burnt fraction of 0.5 %
- * the steps run FIRE_KERNEL_WARP_DENSE with strips of ky = min(ky, 60/sr_y)
- * atmospheric rows; below 0.25 % the default strips come back.
+ * the context goes by FIRE_KERNEL_WARP_DENSE with strips of ky = min(ky, 60/sr_y)
+ * atmospheric rows; below 0.25 % by its strips before.  Strips that the caller
+ * set are launched so; for fire_init's default both names stand for the same
+ * launches (fire_get_launch).
  *   fire_set_adaptive(ctx, 1) turns it on with the current warp strips as
  *     the default shape (FIRE_ERR_ARG unless the context is FIRE_FP32 on
  *     FIRE_KERNEL_WARP or FIRE_KERNEL_WARP_DENSE with the subcell scheme);

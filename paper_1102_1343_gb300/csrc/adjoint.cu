@@ -1633,6 +1633,11 @@ int run_adjoint(fire_ctx *c, int nsteps, double dt, const void *u, const void *v
         return FIRE_OK;
     }
 
+    // the reverse steps need psi alone of the recomputed states: the kernels
+    // that can leave out the rest do (the adjoint of 100 steps of 510^2 nodes
+    // with moisture, FP32: 6.85 -> 6.04 ms; of 60 of 370x290: 4.33 -> 4.08)
+    const bool psi_alone = variant == FIRE_KERNEL_WARP || variant == FIRE_KERNEL_TILE;
+
     // lambda ping-pongs between lam and lam + n, starting in lam; the
     // parameter sums are four fields of n doubles (FP64), or of n
     // compensated float pairs in the same bytes (FP32), turned into doubles
@@ -1643,7 +1648,7 @@ int run_adjoint(fire_ctx *c, int nsteps, double dt, const void *u, const void *v
     static_assert(sizeof(typename GAcc<T>::t) == sizeof(double), "sums in place of doubles");
     ADJ_CHECK(cudaMemsetAsync(lam, 0, n * E, st));
     ADJ_CHECK(cudaMemsetAsync(gm, 0, 4 * n * sizeof(double), st));
-    ADJ_CHECK(cudaMemsetAsync(Fs, 0, 2 * n * E, st));
+    if (!psi_alone) ADJ_CHECK(cudaMemsetAsync(Fs, 0, 2 * n * E, st));
 
     // d(coefficients)/d(M_f) per class at the class moisture, and per node at
     // the node's moisture
@@ -1738,7 +1743,8 @@ int run_adjoint(fire_ctx *c, int nsteps, double dt, const void *u, const void *v
             ADJ_CHECK(cudaFuncSetAttribute(k_adj_step<T>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)rev_smem_bytes<T>(FIRE_MAX_CLASSES)));
-            // all of the unified L1 as shared memory: four tiles per SM
+            // (57 KB a tile; two tiles per SM, which 57 registers of 512 threads
+            // allow, where none end early)
             ADJ_CHECK(cudaFuncSetAttribute(k_adj_step<T>,
                                            cudaFuncAttributePreferredSharedMemoryCarveout, 100));
             if (devid >= 0) rev_attr[devid] = true;
@@ -1777,11 +1783,6 @@ int run_adjoint(fire_ctx *c, int nsteps, double dt, const void *u, const void *v
             k_adj_finish<T><<<grid, kAdjThreads, 0, cs>>>(b);
         }
     };
-
-    // the reverse steps need psi alone of the recomputed states: the kernels
-    // that can leave out the rest do (the adjoint of 100 steps of 510^2 nodes
-    // with moisture, FP32: 6.85 -> 6.04 ms; of 60 of 370x290: 4.33 -> 4.08)
-    const bool psi_alone = variant == FIRE_KERNEL_WARP || variant == FIRE_KERNEL_TILE;
 
     // One segment: ring slot 0 holds its checkpoint and tseg its step times,
     // so every segment of a given length issues the same launches: the

@@ -68,9 +68,6 @@ template <>
 __device__ __forceinline__ Dual constant<Dual>(double x) { return mk(x, 0.0); }
 
 __device__ __forceinline__ double from_lane(double x, int l) { return __shfl_sync(0xffffffffu, x, l); }
-__device__ __forceinline__ Dual from_lane(Dual x, int l) {
-    return mk(__shfl_sync(0xffffffffu, x.v, l), __shfl_sync(0xffffffffu, x.d, l));
-}
 
 // what the chain takes from the class alone
 struct ClassTerms {

@@ -163,7 +163,8 @@ __global__ void __launch_bounds__(kMarchThreads, MarchOccupancy<T>::blocks)
 
 // the warp form: the CTA's warps share one item, its member's arguments in
 // shared memory.  One CTA per SM fewer than k_fire_warp: at 80 registers this
-// kernel spills 176 bytes (28 at 96): 24 members of 26..130 cells square, 40
+// kernel spills 176 bytes (8 at 96, 104 where it holds the row loops of even and
+// odd widths): 24 members of 26..130 cells square, 40
 // steps, 14.35 ms with six CTAs, 13.69 with five (17.8 with the former kernel)
 template <typename T, int MODE, int WIDTH>
 __global__ void __launch_bounds__(32 * kRowWarps, (row_ctas<T, MODE>()) - 1)
@@ -238,7 +239,6 @@ struct fire_ensemble {
     double g_dt = 0;
     int g_grid = 0;
     size_t g_smem = 0;
-    const void *g_first_u = nullptr;
 };
 
 namespace {

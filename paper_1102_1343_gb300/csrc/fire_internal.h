@@ -88,9 +88,9 @@ struct StepArgs {
 
 // A launch that may start while the kernel before it on the stream still runs
 // (programmatic dependent launch): each of these kernels lets its dependents
-// start at once and waits for what it depends on itself before it touches
-// memory (chain_begin), so that one kernel's launch and the filling of the SMs
-// overlap the end of the one before.  Only for chains of the library's own
+// start at once (chain_go) and waits for what it depends on itself before it
+// touches what a step writes (chain_wait), so that one kernel's launch, its tables
+// and the filling of the SMs overlap the end of the one before.  Only for chains of the library's own
 // kernels (chained); after anything else the launch is an ordinary one.
 template <typename... P, typename... A>
 cudaError_t launch_chained(bool chained, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
