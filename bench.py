@@ -544,7 +544,7 @@ def bench_burning(pkg, dev, steps):
     3 km, about 40 % of the domain burnt from the start): cell-steps/s and the
     roofline fraction of the step kernel where most warps run the
     fuel-fraction quadrature and the ignition-time path, with fire_init's
-    default (the adaptive choice between the two warp-strip kernels) and
+    default and
     then with the kernel the autotuner picks there."""
     import torch
     from paper_1102_1343_gb300 import synth
@@ -709,9 +709,10 @@ def bench_adjoint(pkg, dev, ckpt=20):
         rec["reverse_step"] = {"us": us, "bytes_per_node": b_node, "achieved_gbs": gbs,
                                "frac_of_hbm": gbs / peak, "peak_source": f"{peak_kind} hbm_gbs",
                                "kernel": "k_adj_step<float> (one launch)" if prec == "fp32" else
-                               "k_adj_stage1/vjp_star/vjp_n/finish<double> (four launches)",
+                               "k_adj_seed/stage1/vjp_star/vjp_n/finish<double> (five launches)",
                                "note": "estimated as (every-state-kept call - plain forward) / "
-                                       "steps; the step's working set fits in L2"}
+                                       "steps; the step's working set fits in L2, and nodes without an "
+                                       "adjoint leave most of the bytes out"}
         out[prec] = rec
         m.close()
     base = out["fp64"]["plain_forward"]["value"]

@@ -28,8 +28,9 @@
 // (meshes below 2^31 nodes).
 //
 // What bounds it: instruction issue.  A row of a warp takes 485 warp
-// instructions, 160 of them the method's arithmetic, at ~70 % issue with 24
-// warps per SM (DRAM at 20 % of its rate).  The form before it, a warp
+// instructions, 160 of them the method's arithmetic, at 60 % issue with 21 of 24
+// warps active per SM (DRAM at 25 % of its rate; 4000^2 nodes, strips of 100
+// rows).  The form before it, a warp
 // marching alone with its rows in registers, took 515 at 58 % with the 12
 // warps its 159 registers allowed, and one strip's rows ran one after the
 // other.  Measured, us per FP32 step, before and now (GB300): 8200^2 nodes,
