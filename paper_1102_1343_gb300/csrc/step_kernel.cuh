@@ -646,7 +646,7 @@ __global__ void __launch_bounds__(kIgnThreads) k_ignite(const IgniteArgs a) {
             }
             double u, d;
             const double pg = ignition_distance(s, x, y, u, d);
-            if (pe > T(0) && le0(pg)) {
+            if (pe > T(0) && __double_as_longlong(pg) <= 0) {  // (pg is a number: at most 0)
                 if (!read) {
                     ti = a.tign[g];
                     read = true;
