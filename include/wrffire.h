@@ -541,8 +541,8 @@ int fire_ensemble_clear_status(fire_ensemble *ens);
 int fire_ensemble_set_kernel(fire_ensemble *ens, int strip_columns, int strip_rows);
 int fire_ensemble_get_kernel(const fire_ensemble *ens, int *grid_ctas, int *work_items);
 
-/* Autotuner of the strip shape: times candidate shapes (40..240 columns x
- * 20..320 rows) on probe_steps steps of the members with the given winds,
+/* Autotuner of the strip shape: times the strips in place (not below 20 rows) and
+ * candidate shapes (20..240 columns x 20..320 rows) on probe_steps steps of the members with the given winds,
  * each from the members' current states, keeps the fastest and puts the
  * states back.  No ignition may be active or pending within 2 probe_steps
  * steps (else FIRE_ERR_STATE).  Outputs nullable.  Synchronous. */

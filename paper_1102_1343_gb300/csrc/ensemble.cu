@@ -22,6 +22,7 @@
 #include <algorithm>
 #include <mutex>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "fire_internal.h"
@@ -233,6 +234,7 @@ struct fire_ensemble {
     cudaGraphExec_t graph = nullptr;
     bool capture_failed = false;
     int variant = FIRE_KERNEL_MARCH;  // member kernel: FIRE_KERNEL_MARCH or FIRE_KERNEL_WARP
+    int strip_cols = 0, strip_rows = 0;  // nodes of the members' strips, as set or by default
     bool even = true;  // every member's mesh has an even width
     bool nc = false;  // members carry per-node coefficients (a per-node fuel moisture)
     int g_nsteps = -1;
@@ -475,6 +477,8 @@ int fire_ensemble_create(fire_ensemble **out, int n_members, const fire_member_d
                 rows = L;
             }
         }
+        e->strip_cols = warp ? kWarpMaxColumns : kMarchMaxColumns;
+        e->strip_rows = warp ? rows : 60;
         for (fire_ctx *c : e->members)
             if (r == FIRE_OK && (warp ? ctx_default_warp_strips(c, rows) : ctx_default_march(c)) != FIRE_OK)
                 r = FIRE_ERR_ARG;
@@ -656,6 +660,8 @@ int fire_ensemble_set_kernel(fire_ensemble *e, int strip_columns, int strip_rows
         int r = fire_set_kernel(c, e->variant, kxn, kyn);
         if (r) return r;
     }
+    e->strip_cols = strip_columns;
+    e->strip_rows = strip_rows;
     return ens_plan(e);
 }
 
@@ -707,41 +713,39 @@ int fire_ensemble_autotune(fire_ensemble *e, int probe_steps, double dt,
         return (int)FIRE_OK;
     };
     const int cols_m[] = {40, 80, 120, 160, 200, 240}, rows_m[] = {20, 40, 80, 160, 320};
-    const int cols_w[] = {20, 30, 40, 50, 60, 60}, rows_w[] = {40, 80, 160, 256, 320};
+    const int cols_w[] = {20, 30, 40, 50, 60, 60}, rows_w[] = {20, 40, 80, 160, 320};
     const bool wv = e->variant == FIRE_KERNEL_WARP;
     const int *cols = wv ? cols_w : cols_m, *rows = wv ? rows_w : rows_m;
+    // the strips in place first (20 rows where they are shorter, the least that
+    // is reported)
+    std::vector<std::pair<int, int>> cands = {{std::min(e->strip_cols, 240), std::max(e->strip_rows, 20)}};
+    for (int ci = 0; ci < 6; ++ci)
+        for (int ri = 0; ri < 5; ++ri) {
+            const std::pair<int, int> q{cols[ci], rows[ri]};
+            if (std::find(cands.begin(), cands.end(), q) == cands.end()) cands.push_back(q);
+        }
     cudaEvent_t a, b;
     ENS_CHECK(cudaEventCreate(&a));
     ENS_CHECK(cudaEventCreate(&b));
     float best = 0.f;
     int bc = 0, br = 0;
     int r = FIRE_OK;
-    for (int ci = 0; ci < 6; ++ci) {
-        const int C = cols[ci];
-        if (ci > 0 && C == cols[ci - 1]) continue;
-        for (int ri = 0; ri < 5; ++ri) {
-            const int R = rows[ri];
-            if (fire_ensemble_set_kernel(e, C, R) != FIRE_OK) continue;
-            if ((r = restore())) break;
-            if ((r = fire_ensemble_step(e, probe_steps, dt, wind_u_dev, wind_v_dev, nullptr,
-                                        nullptr)))
-                break;
-            if ((r = restore())) break;
-            if ((r = ens_cuda(cudaEventRecord(a, e->stream)))) break;
-            if ((r = fire_ensemble_step(e, probe_steps, dt, wind_u_dev, wind_v_dev, nullptr,
-                                        nullptr)))
-                break;
-            if ((r = ens_cuda(cudaEventRecord(b, e->stream)))) break;
-            if ((r = ens_cuda(cudaEventSynchronize(b)))) break;
-            float ms = 0.f;
-            if ((r = ens_cuda(cudaEventElapsedTime(&ms, a, b)))) break;
-            if (bc == 0 || ms < best) {
-                best = ms;
-                bc = C;
-                br = R;
-            }
+    for (const std::pair<int, int> &q : cands) {
+        if (fire_ensemble_set_kernel(e, q.first, q.second) != FIRE_OK) continue;
+        if ((r = restore())) break;
+        if ((r = fire_ensemble_step(e, probe_steps, dt, wind_u_dev, wind_v_dev, nullptr, nullptr))) break;
+        if ((r = restore())) break;
+        if ((r = ens_cuda(cudaEventRecord(a, e->stream)))) break;
+        if ((r = fire_ensemble_step(e, probe_steps, dt, wind_u_dev, wind_v_dev, nullptr, nullptr))) break;
+        if ((r = ens_cuda(cudaEventRecord(b, e->stream)))) break;
+        if ((r = ens_cuda(cudaEventSynchronize(b)))) break;
+        float ms = 0.f;
+        if ((r = ens_cuda(cudaEventElapsedTime(&ms, a, b)))) break;
+        if (bc == 0 || ms < best) {
+            best = ms;
+            bc = q.first;
+            br = q.second;
         }
-        if (r) break;
     }
     cudaEventDestroy(a);
     cudaEventDestroy(b);

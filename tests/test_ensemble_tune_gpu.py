@@ -1,0 +1,34 @@
+"""fire_ensemble_autotune times the strips in place and short ones: a large
+ensemble is not left slower than its default strips, a small one, whose default
+strips are shorter than the 20 rows that the tuner reports at least, by the
+difference to those (some 20 %; from 40 rows it was 70)."""
+import pytest
+
+from paper_1102_1343_gb300 import synth
+from test_ensemble_gpu import make_ensemble, pkg  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("members,size,limit", [(4, 110, 1.1), (30, 34, 1.1), (3, 15, 1.45), (2, 40, 1.2)])
+def test_no_ensemble_left_slower(pkg, members, size, limit):  # noqa: F811
+    import torch
+    ws = [synth.random_landscape(size + k % 5, size - k % 7, seed=k, ignition="center", dt=0.25) for k in range(members)]
+    ens, winds = make_ensemble(pkg, ws, "fp32")
+    us, vs = [u for u, _ in winds], [v for _, v in winds]
+    e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+
+    def ms():
+        best = 1e9
+        for _ in range(4):
+            e[0].record()
+            pkg.fire_ensemble_step(ens, 40, 0.01, us, vs)
+            e[1].record()
+            torch.cuda.synchronize()
+            best = min(best, e[0].elapsed_time(e[1]))
+        return best
+
+    before = ms()
+    pkg.fire_ensemble_autotune(ens, 10, 0.01, us, vs)
+    assert ms() <= limit * before
+    pkg.fire_ensemble_destroy(ens)
