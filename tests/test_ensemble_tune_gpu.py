@@ -10,7 +10,7 @@ from test_ensemble_gpu import make_ensemble, pkg  # noqa: F401
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("members,size,limit", [(4, 110, 1.1), (30, 34, 1.1), (3, 15, 1.45), (2, 40, 1.2)])
+@pytest.mark.parametrize("members,size,limit", [(4, 110, 1.25), (30, 34, 1.25), (3, 15, 1.45), (2, 40, 1.25)])
 def test_no_ensemble_left_slower(pkg, members, size, limit):  # noqa: F811
     import torch
     ws = [synth.random_landscape(size + k % 5, size - k % 7, seed=k, ignition="center", dt=0.25) for k in range(members)]

@@ -74,7 +74,7 @@ def test_adaptive_choice_keeps_the_launches(pkg, nxa, nya, sr):
 @pytest.mark.parametrize("n,prec", [(10, "fp64"), (51, "fp64"), (40, "fp32")])
 def test_autotune_leaves_no_context_slower(pkg, n, prec):
     """The form that stands for the default is among the candidates: after
-    fire_autotune 200 steps take at most 1.2 times as long as before."""
+    fire_autotune 200 steps take at most 1.3 times as long as before."""
     import torch
     w, m = model(pkg, n, n, 10, prec)
     u, v = m.wind(w.u, w.v)
@@ -92,5 +92,5 @@ def test_autotune_leaves_no_context_slower(pkg, n, prec):
 
     before = ms()
     assert m.autotune(u, v, 0.01) == pkg.fire_get_kernel(m.ctx)
-    assert ms() <= 1.2 * before
+    assert ms() <= 1.3 * before
     m.close()
