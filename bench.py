@@ -544,8 +544,7 @@ def bench_burning(pkg, dev, steps):
     3 km, about 40 % of the domain burnt from the start): cell-steps/s and the
     roofline fraction of the step kernel where most warps run the
     fuel-fraction quadrature and the ignition-time path, with fire_init's
-    default and
-    then with the kernel the autotuner picks there."""
+    default and then with the kernel the autotuner picks there."""
     import torch
     from paper_1102_1343_gb300 import synth
     w = synth.burning_fire_8200()
